@@ -23,6 +23,7 @@ points keep the C names:
                           gradient (App. F, Algorithm 1)
 """
 import ctypes
+import struct
 
 import torch
 
@@ -58,14 +59,23 @@ def lib():
     return _lib.load()
 
 
+# The marshalling below runs on every call of a decode loop, where a call's
+# kernels take a few microseconds, so it is kept short: addresses go to ctypes
+# as plain integers, the host structs as packed bytes (0.3 us against 1.5 us
+# for a ctypes struct), and the current stream's handle is read without
+# building a Stream object (0.2 us against 2.9 us).  A step of five
+# calls (cache update, four layers' attention) over three short sequences, bound
+# by the host, went from 152 to 94 us.
 def _p(t):
-    return ctypes.c_void_p(0 if t is None else t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if torch.cuda.is_initialized():
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _check(code, where):
@@ -77,6 +87,11 @@ def _dev(t):
     if not t.is_cuda:
         raise ValueError("expected a CUDA tensor")
     return t.device
+
+
+def _on_gpu(t):
+    if not t.is_cuda:
+        raise ValueError("expected a CUDA tensor")
 
 
 def new_status(device):
@@ -95,22 +110,42 @@ def workspace(nbytes, device):
     return torch.zeros(max(int(nbytes), 256), dtype=torch.uint8, device=device)
 
 
+def _pool_fields(pool):
+    """(base, layers, pages, Hkv, page size, D) of a checked pool."""
+    shape = pool.shape
+    if pool.dtype != torch.bfloat16 or len(shape) != 6 or shape[2] != 2 or not pool.is_contiguous():
+        raise ValueError("pool must be contiguous bf16 [layers][pages][2][Hkv][16][D]")
+    layers, pages, _, heads, page_size, head_dim = shape
+    return pool.data_ptr(), layers, pages, heads, page_size, head_dim
+
+
 def paged_kv(pool):
     """umim_paged_kv for a bf16 pool shaped [layers][pages][2][Hkv][16][D]."""
-    if pool.dtype != torch.bfloat16 or pool.dim() != 6 or pool.shape[2] != 2 or not pool.is_contiguous():
-        raise ValueError("pool must be contiguous bf16 [layers][pages][2][Hkv][16][D]")
-    return PagedKVC(pool.data_ptr(), pool.shape[0], pool.shape[1], pool.shape[3], pool.shape[4], pool.shape[5])
+    return PagedKVC(*_pool_fields(pool))
+
+
+# the layouts of umim_paged_kv and umim_merge_weights (native alignment)
+_pack_kv = struct.Struct("@P5i4x").pack
+_pack_weights = struct.Struct("@9P2if4x").pack
+_WEIGHTS = ("w_kv", "b_kv", "ln_kv_gamma", "ln_kv_beta", "query", "w_o", "b_o", "ln_o_gamma", "ln_o_beta")
+
+
+def _weight_fields(w):
+    if isinstance(w, dict):
+        tensors = [w[k] for k in _WEIGHTS]
+        rest = (int(w["d_model"]), int(w["n_heads"]), float(w["ln_eps"]))
+    else:
+        tensors = [getattr(w, k) for k in _WEIGHTS]
+        rest = (int(w.d_model), int(w.n_heads), float(w.ln_eps))
+    for k, t in zip(_WEIGHTS, tensors):
+        if t.dtype != torch.bfloat16 or not t.is_contiguous():
+            raise ValueError(f"merge weight {k} must be contiguous bf16")
+    return [t.data_ptr() for t in tensors], rest
 
 
 def merge_weights_c(w):
-    g = (lambda k: getattr(w, k)) if not isinstance(w, dict) else (lambda k: w[k])
-    names = ("w_kv", "b_kv", "ln_kv_gamma", "ln_kv_beta", "query", "w_o", "b_o", "ln_o_gamma", "ln_o_beta")
-    for k in names:
-        t = g(k)
-        if t.dtype != torch.bfloat16 or not t.is_contiguous():
-            raise ValueError(f"merge weight {k} must be contiguous bf16")
-    return MergeWeightsC(*[g(k).data_ptr() for k in names], int(g("d_model")), int(g("n_heads")),
-                         float(g("ln_eps")))
+    ptrs, rest = _weight_fields(w)
+    return MergeWeightsC(*ptrs, *rest)
 
 
 # ---------------------------------------------------------------------------
@@ -142,18 +177,19 @@ def umim_decode_attention_workspace_size(batch, n_q_heads, n_kv_heads, head_dim)
 def umim_merge_spans(embeddings, token_ids, span_offsets, weights, surrogates=None, workspace_buf=None,
                      dev_status=None, stream=None):
     """Surrogate embeddings z (fp32 [S][d]) of the spans in CSR form."""
-    dev = _dev(embeddings)
-    d = embeddings.shape[1]
+    _on_gpu(embeddings)
+    shape = embeddings.shape
+    vocab, d = shape[0], shape[1]
     S = span_offsets.numel() - 1
     T = token_ids.numel()
     if surrogates is None:
-        surrogates = torch.empty((S, d), dtype=torch.float32, device=dev)
+        surrogates = torch.empty((S, d), dtype=torch.float32, device=embeddings.device)
     if workspace_buf is None:
-        workspace_buf = workspace(umim_merge_spans_workspace_size(T, S, d), dev)
-    wc = merge_weights_c(weights)
-    code = lib().umim_merge_spans(_p(embeddings), embeddings.shape[0], _p(token_ids), T, _p(span_offsets), S,
-                                  ctypes.byref(wc), _p(surrogates), _p(workspace_buf), workspace_buf.numel(),
-                                  _p(dev_status), _stream(stream))
+        workspace_buf = workspace(umim_merge_spans_workspace_size(T, S, d), embeddings.device)
+    ptrs, rest = _weight_fields(weights)
+    code = lib().umim_merge_spans(embeddings.data_ptr(), vocab, token_ids.data_ptr(), T, span_offsets.data_ptr(), S,
+                                  _pack_weights(*ptrs, *rest), surrogates.data_ptr(), workspace_buf.data_ptr(),
+                                  workspace_buf.numel(), _p(dev_status), _stream(stream))
     _check(code, "umim_merge_spans")
     return surrogates
 
@@ -163,9 +199,11 @@ def umim_build_compressed(embeddings, token_ids, span_offsets, span_start, span_
                           dev_status=None, stream=None):
     """(out_embeds [rows][d] bf16, position_ids [rows], cu_seqlens [B+1]); the
     first cu_seqlens[-1] rows are the packed compressed prompts."""
-    dev = _dev(embeddings)
+    _on_gpu(embeddings)
+    dev = embeddings.device
     B, L = token_ids.shape
-    d = embeddings.shape[1]
+    shape = embeddings.shape
+    vocab, d = shape[0], shape[1]
     S = span_start.numel()
     if out_embeds is None:
         out_embeds = torch.empty((B * L, d), dtype=torch.bfloat16, device=dev)
@@ -175,7 +213,7 @@ def umim_build_compressed(embeddings, token_ids, span_offsets, span_start, span_
         cu_seqlens = torch.empty(B + 1, dtype=torch.int32, device=dev)
     if workspace_buf is None:
         workspace_buf = workspace(umim_build_compressed_workspace_size(B, S), dev)
-    code = lib().umim_build_compressed(_p(embeddings), embeddings.shape[0], d, _p(token_ids), B, L,
+    code = lib().umim_build_compressed(_p(embeddings), vocab, d, _p(token_ids), B, L,
                                        _p(span_offsets), _p(span_start), _p(span_len), S, _p(surrogates),
                                        _p(out_embeds), out_embeds.shape[0], _p(position_ids), _p(cu_seqlens),
                                        _p(workspace_buf), workspace_buf.numel(), _p(dev_status), _stream(stream))
@@ -190,24 +228,23 @@ def umim_kv_rollback(pool, block_table, seq_lens, span_offsets, span_start, span
     (device int32 [B*max_pages], -1 terminated).  With rope_inv_freq (device
     fp32 [rotary_dim/2]) moved keys are re-rotated to their compressed
     positions (umim_kv_rollback_rope)."""
-    dev = _dev(pool)
-    kv = paged_kv(pool)
+    _on_gpu(pool)
+    kv = _pool_fields(pool)
     B, max_pages = block_table.shape
     S = span_start.numel()
     if freed_pages is None:
-        freed_pages = torch.empty(max(1, B * max_pages), dtype=torch.int32, device=dev)
+        freed_pages = torch.empty(max(1, B * max_pages), dtype=torch.int32, device=pool.device)
     if workspace_buf is None:
-        workspace_buf = workspace(umim_kv_rollback_workspace_size(B, S, max_pages, kv.n_layers, kv.n_kv_heads,
-                                                                  kv.head_dim), dev)
+        workspace_buf = workspace(umim_kv_rollback_workspace_size(B, S, max_pages, kv[1], kv[3], kv[5]), pool.device)
     if rope_inv_freq is None:
-        code = lib().umim_kv_rollback(ctypes.byref(kv), _p(block_table), max_pages, _p(seq_lens), B,
+        code = lib().umim_kv_rollback(_pack_kv(*kv), _p(block_table), max_pages, _p(seq_lens), B,
                                       _p(span_offsets), _p(span_start), _p(span_len), S, _p(surrogate_k),
                                       _p(surrogate_v), _p(freed_pages), _p(workspace_buf), workspace_buf.numel(),
                                       _p(dev_status), _stream(stream))
         _check(code, "umim_kv_rollback")
     else:
-        rd = kv.head_dim if rotary_dim is None else int(rotary_dim)
-        code = lib().umim_kv_rollback_rope(ctypes.byref(kv), _p(block_table), max_pages, _p(seq_lens), B,
+        rd = kv[5] if rotary_dim is None else int(rotary_dim)
+        code = lib().umim_kv_rollback_rope(_pack_kv(*kv), _p(block_table), max_pages, _p(seq_lens), B,
                                            _p(span_offsets), _p(span_start), _p(span_len), S, _p(surrogate_k),
                                            _p(surrogate_v), _p(rope_inv_freq), rd, _p(freed_pages),
                                            _p(workspace_buf), workspace_buf.numel(), _p(dev_status), _stream(stream))
@@ -218,9 +255,9 @@ def umim_kv_rollback(pool, block_table, seq_lens, span_offsets, span_start, span
 def umim_kv_append(pool, block_table, seq_lens, new_k, new_v, new_pages=None, dev_status=None, stream=None):
     """In-place append of one entry per layer to every sequence (new_k/new_v
     [B][n_layers][Hkv][D] bf16; new_pages [B] int32, read at page boundaries)."""
-    kv = paged_kv(pool)
+    kv = _pack_kv(*_pool_fields(pool))
     B, max_pages = block_table.shape
-    code = lib().umim_kv_append(ctypes.byref(kv), _p(block_table), max_pages, _p(seq_lens), B, _p(new_k),
+    code = lib().umim_kv_append(kv, _p(block_table), max_pages, _p(seq_lens), B, _p(new_k),
                                 _p(new_v), _p(new_pages), _p(dev_status), _stream(stream))
     _check(code, "umim_kv_append")
 
@@ -232,12 +269,12 @@ def umim_decode_append_merge(pool, block_table, seq_lens, new_k, new_v, new_page
     or, where merge_k[b] = k > 0, write surrogate row merge_row[b] in place of
     the last k entries (the new one included).  Returns released [B] int32
     (the page a merge freed, or -1)."""
-    kv = paged_kv(pool)
+    kv = _pack_kv(*_pool_fields(pool))
     B, max_pages = block_table.shape
     if released is None:
         released = torch.empty(B, dtype=torch.int32, device=pool.device)
     n_rows = 0 if surrogate_k is None else surrogate_k.shape[0]
-    code = lib().umim_decode_append_merge(ctypes.byref(kv), _p(block_table), max_pages, _p(seq_lens), B, _p(new_k),
+    code = lib().umim_decode_append_merge(kv, _p(block_table), max_pages, _p(seq_lens), B, _p(new_k),
                                           _p(new_v), _p(new_pages), _p(merge_k), _p(merge_row), n_rows,
                                           _p(surrogate_k), _p(surrogate_v), _p(released), _p(dev_status),
                                           _stream(stream))
@@ -248,17 +285,17 @@ def umim_decode_append_merge(pool, block_table, seq_lens, new_k, new_v, new_page
 def umim_decode_attention(q, pool, layer, block_table, seq_lens, scale=0.0, out=None, workspace_buf=None,
                           dev_status=None, stream=None):
     """out [B][Hq][D] bf16 = GQA attention of q over the paged cache."""
-    dev = _dev(q)
-    kv = paged_kv(pool)
+    _on_gpu(q)
+    kv = _pool_fields(pool)
     B, Hq, D = q.shape
-    max_pages = block_table.shape[1]
     if out is None:
         out = torch.empty_like(q)
     if workspace_buf is None:
-        workspace_buf = workspace(umim_decode_attention_workspace_size(B, Hq, kv.n_kv_heads, D), dev)
-    code = lib().umim_decode_attention(_p(q), Hq, ctypes.byref(kv), layer, _p(block_table), max_pages,
-                                       _p(seq_lens), B, float(scale), _p(out), _p(workspace_buf),
-                                       workspace_buf.numel(), _p(dev_status), _stream(stream))
+        workspace_buf = workspace(umim_decode_attention_workspace_size(B, Hq, kv[3], D), q.device)
+    code = lib().umim_decode_attention(q.data_ptr(), Hq, _pack_kv(*kv), layer, block_table.data_ptr(),
+                                       block_table.shape[1], seq_lens.data_ptr(), B, float(scale), out.data_ptr(),
+                                       workspace_buf.data_ptr(), workspace_buf.numel(), _p(dev_status),
+                                       _stream(stream))
     _check(code, "umim_decode_attention")
     return out
 
@@ -277,22 +314,22 @@ def umim_decode_layer_step(q, pool, layer, block_table, seq_lens, new_k, new_v, 
     surrogate_v are [rows][Hkv][D].  commit=True on the step's last layer
     records the new lengths, opened pages and released pages.  workspace_buf
     must be zeroed before its first use (workspace() zeroes it)."""
-    dev = _dev(q)
-    kv = paged_kv(pool)
+    _on_gpu(q)
+    kv = _pool_fields(pool)
     B, Hq, D = q.shape
-    for t in (new_k, new_v):
-        if t.dtype != torch.bfloat16 or t.dim() != 3 or t.shape[0] != B or t.stride(2) != 1 or \
-                t.stride(1) != t.shape[2]:
+    stride = new_k.stride()
+    for t, st in ((new_k, stride), (new_v, new_v.stride())):
+        if t.dtype != torch.bfloat16 or len(st) != 3 or t.shape[0] != B or st[2] != 1 or st[1] != t.shape[2]:
             raise ValueError("new_k / new_v must be bf16 [B][Hkv][D] with contiguous rows")
-    if new_k.stride(0) != new_v.stride(0):
-        raise ValueError("new_k and new_v must have the same row stride")
+        if st[0] != stride[0]:
+            raise ValueError("new_k and new_v must have the same row stride")
     if out is None:
         out = torch.empty_like(q)
     if workspace_buf is None:
-        workspace_buf = workspace(umim_decode_layer_step_workspace_size(B, kv.n_kv_heads, D), dev)
+        workspace_buf = workspace(umim_decode_layer_step_workspace_size(B, kv[3], D), q.device)
     n_rows = 0 if surrogate_k is None else surrogate_k.shape[0]
-    code = lib().umim_decode_layer_step(_p(q), Hq, ctypes.byref(kv), layer, _p(block_table), block_table.shape[1],
-                                        _p(seq_lens), B, _p(new_k), _p(new_v), new_k.stride(0), _p(new_pages),
+    code = lib().umim_decode_layer_step(_p(q), Hq, _pack_kv(*kv), layer, _p(block_table), block_table.shape[1],
+                                        _p(seq_lens), B, _p(new_k), _p(new_v), stride[0], _p(new_pages),
                                         _p(merge_k), _p(merge_row), n_rows, _p(surrogate_k), _p(surrogate_v),
                                         1 if commit else 0, _p(released), float(scale), _p(out), _p(workspace_buf),
                                         workspace_buf.numel(), _p(dev_status), _stream(stream))
@@ -306,11 +343,11 @@ def umim_decode_attention_static(q, pool, layer, block_table, seq_lens, scale=0.
     allocate GPU memory at call time: the library's fixed scratch array is
     used instead (see include/umim.h for the size limit and the rule that
     overlapping calls must not run concurrently)."""
-    kv = paged_kv(pool)
+    kv = _pack_kv(*_pool_fields(pool))
     B, Hq, D = q.shape
     if out is None:
         out = torch.empty_like(q)
-    code = lib().umim_decode_attention_static(_p(q), Hq, ctypes.byref(kv), layer, _p(block_table),
+    code = lib().umim_decode_attention_static(_p(q), Hq, kv, layer, _p(block_table),
                                               block_table.shape[1], _p(seq_lens), B, float(scale), _p(out),
                                               _p(dev_status), _stream(stream))
     _check(code, "umim_decode_attention_static")

@@ -31,29 +31,31 @@ class PagedKVC(ctypes.Structure):
     ]
 
 
-# name -> (restype, argtypes), exactly as declared in include/umim.h
+# name -> (restype, argtypes), exactly as declared in include/umim.h; a pointer
+# to a host struct is a c_void_p here, which takes byref(struct) as well as the
+# packed bytes of one (the binding packs them: a fraction of a ctypes struct's cost)
 SIGNATURES = {
     "umim_status_string": (ctypes.c_char_p, [ctypes.c_int]),
     "umim_version": (ctypes.c_int, []),
     "umim_merge_spans_workspace_size": (c_size, [c_i64, c_i32, c_i32]),
     "umim_merge_spans": (ctypes.c_int, [c_ptr, c_i64, c_ptr, c_i64, c_ptr, c_i32,
-                                        ctypes.POINTER(MergeWeightsC), c_ptr, c_ptr, c_size, c_ptr, c_ptr]),
+                                        c_ptr, c_ptr, c_ptr, c_size, c_ptr, c_ptr]),
     "umim_build_compressed_workspace_size": (c_size, [c_i32, c_i32]),
     "umim_build_compressed": (ctypes.c_int, [c_ptr, c_i64, c_i32, c_ptr, c_i32, c_i32, c_ptr, c_ptr, c_ptr,
                                              c_i32, c_ptr, c_ptr, c_i64, c_ptr, c_ptr, c_ptr, c_size, c_ptr,
                                              c_ptr]),
     "umim_kv_rollback_workspace_size": (c_size, [c_i32, c_i32, c_i32, c_i32, c_i32, c_i32]),
-    "umim_kv_rollback": (ctypes.c_int, [ctypes.POINTER(PagedKVC), c_ptr, c_i32, c_ptr, c_i32, c_ptr, c_ptr,
+    "umim_kv_rollback": (ctypes.c_int, [c_ptr, c_ptr, c_i32, c_ptr, c_i32, c_ptr, c_ptr,
                                         c_ptr, c_i32, c_ptr, c_ptr, c_ptr, c_ptr, c_size, c_ptr, c_ptr]),
-    "umim_kv_rollback_rope": (ctypes.c_int, [ctypes.POINTER(PagedKVC), c_ptr, c_i32, c_ptr, c_i32, c_ptr, c_ptr,
+    "umim_kv_rollback_rope": (ctypes.c_int, [c_ptr, c_ptr, c_i32, c_ptr, c_i32, c_ptr, c_ptr,
                                              c_ptr, c_i32, c_ptr, c_ptr, c_ptr, c_i32, c_ptr, c_ptr, c_size, c_ptr,
                                              c_ptr]),
-    "umim_kv_append": (ctypes.c_int, [ctypes.POINTER(PagedKVC), c_ptr, c_i32, c_ptr, c_i32, c_ptr, c_ptr, c_ptr,
+    "umim_kv_append": (ctypes.c_int, [c_ptr, c_ptr, c_i32, c_ptr, c_i32, c_ptr, c_ptr, c_ptr,
                                       c_ptr, c_ptr]),
-    "umim_decode_append_merge": (ctypes.c_int, [ctypes.POINTER(PagedKVC), c_ptr, c_i32, c_ptr, c_i32, c_ptr, c_ptr,
+    "umim_decode_append_merge": (ctypes.c_int, [c_ptr, c_ptr, c_i32, c_ptr, c_i32, c_ptr, c_ptr,
                                                 c_ptr, c_ptr, c_ptr, c_i32, c_ptr, c_ptr, c_ptr, c_ptr, c_ptr]),
     "umim_decode_layer_step_workspace_size": (c_size, [c_i32, c_i32, c_i32]),
-    "umim_decode_layer_step": (ctypes.c_int, [c_ptr, c_i32, ctypes.POINTER(PagedKVC), c_i32, c_ptr, c_i32, c_ptr,
+    "umim_decode_layer_step": (ctypes.c_int, [c_ptr, c_i32, c_ptr, c_i32, c_ptr, c_i32, c_ptr,
                                               c_i32, c_ptr, c_ptr, c_i64, c_ptr, c_ptr, c_ptr, c_i32, c_ptr, c_ptr,
                                               c_i32, c_ptr, ctypes.c_float, c_ptr, c_ptr, c_size, c_ptr, c_ptr]),
     "umim_selftest_bounded_wait": (ctypes.c_int, [c_i32, ctypes.c_uint32, c_ptr, c_ptr, c_ptr, c_ptr]),
@@ -75,10 +77,10 @@ SIGNATURES = {
     "umim_distill_soft_ce": (ctypes.c_int, [c_ptr, c_i32, c_ptr, c_i32, c_i32, c_i64, c_ptr, c_ptr, c_i32, c_ptr,
                                             ctypes.c_float, c_ptr, c_ptr, c_ptr, c_ptr, c_size, c_ptr, c_ptr]),
     "umim_decode_attention_workspace_size": (c_size, [c_i32, c_i32, c_i32, c_i32]),
-    "umim_decode_attention": (ctypes.c_int, [c_ptr, c_i32, ctypes.POINTER(PagedKVC), c_i32, c_ptr, c_i32,
+    "umim_decode_attention": (ctypes.c_int, [c_ptr, c_i32, c_ptr, c_i32, c_ptr, c_i32,
                                              c_ptr, c_i32, ctypes.c_float, c_ptr, c_ptr, c_size, c_ptr,
                                              c_ptr]),
-    "umim_decode_attention_static": (ctypes.c_int, [c_ptr, c_i32, ctypes.POINTER(PagedKVC), c_i32, c_ptr, c_i32,
+    "umim_decode_attention_static": (ctypes.c_int, [c_ptr, c_i32, c_ptr, c_i32, c_ptr, c_i32,
                                                     c_ptr, c_i32, ctypes.c_float, c_ptr, c_ptr, c_ptr]),
     "umim_debug_build": (ctypes.c_int, []),
     "umim_debug_site_name": (ctypes.c_char_p, [c_i32]),

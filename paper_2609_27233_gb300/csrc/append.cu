@@ -57,10 +57,6 @@ __device__ __forceinline__ uint4 ld_nc_v4(const uint16_t *p) {
   return v;
 }
 
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 template <int D>
 __global__ void __launch_bounds__(kAppendThreads) decode_update_kernel(AppendArgs a, int C) {
   griddep_wait();
@@ -94,7 +90,7 @@ __global__ void __launch_bounds__(kAppendThreads) decode_update_kernel(AppendArg
     s_k = k;
   }
   __syncthreads();
-  cluster_sync();   // every CTA of this sequence has read L, k and the pages
+  cluster_sync_all();   // every CTA of this sequence has read L, k and the pages
   const int page = s_page, slot = s_slot, row = s_row, L = s_L, k = s_k;
   if (page < 0) return;   // this sequence is left unchanged
 
@@ -159,21 +155,9 @@ umim_status launch_update(const AppendArgs &a, int head_dim, int32_t B, cudaStre
   int C = (total + kAppendThreads * kUnroll - 1) / (kAppendThreads * kUnroll);
   C = C < 1 ? 1 : (C > kMaxCluster ? kMaxCluster : C);
   auto kern = head_dim == 128 ? decode_update_kernel<128> : decode_update_kernel<64>;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(B * C));
-  cfg.blockDim = dim3(kAppendThreads);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = (unsigned)C;
-  attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
   trace_mark(stream, label);
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a, C);
+  const cudaError_t e =
+      launch_pdl_cluster(kern, dim3((unsigned)(B * C)), dim3(kAppendThreads), (unsigned)C, 0, stream, a, C);
   trace_mark(stream, nullptr);
   return e == cudaSuccess ? UMIM_OK : UMIM_ERR_CUDA;
 }

@@ -329,11 +329,6 @@ __global__ void ce_prep_kernel(CeArgs a) {
   }
 }
 
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
 __device__ __forceinline__ uint32_t cluster_idx() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(r));
@@ -344,9 +339,6 @@ __device__ __forceinline__ uint32_t cluster_count() {
   asm volatile("mov.u32 %0, %%nclusterid.x;" : "=r"(r));
   return r;
 }
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar,
                                           uint64_t policy) {
   asm volatile(
@@ -354,12 +346,6 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
           smem_u32(dst)),
       "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(policy)
       : "memory");
-}
-
-__device__ __forceinline__ uint32_t cluster_size() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-  return r;
 }
 
 // The hardware's approximate base-2 exponential, logarithm and reciprocal
@@ -499,11 +485,6 @@ __device__ __forceinline__ void store8(uint16_t *row, int64_t e, int V, const fl
 // armed (arrive + expected bytes) by thread 0 one row ahead, right after the
 // previous phase of that buffer completed, so its byte count never runs
 // negative.
-__device__ __forceinline__ uint32_t peer_addr(const void *local, uint32_t rank) {
-  uint32_t ra;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(smem_u32(local)), "r"(rank));
-  return ra;
-}
 __device__ __forceinline__ void st_async_f4(uint32_t raddr, float4 v, uint32_t rbar) {
   asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
                    raddr),

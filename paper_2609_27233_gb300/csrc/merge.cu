@@ -37,12 +37,21 @@ __device__ __forceinline__ void bf16x8_to_float(uint4 u, float *f) {
   }
 }
 
-template <typename OutT>
+// Whether a value did not fit fp16: one word per CTA of each kernel that checks
+// (GEMM1, pooling, W_o conversion, GEMM2), written by every CTA on every call,
+// so that no kernel has to clear them first.
+constexpr int kFlagCtas = 1024;   // CTAs per kernel, at most
+enum FlagKernel { kFlagGemm1, kFlagPool, kFlagWo, kFlagGemm2, kFlagKernels };
+struct RangeFlags {
+  int32_t *words;              // [kFlagKernels][kFlagCtas]
+  int32_t n[kFlagKernels];     // CTAs of each kernel of this call (0: not launched)
+};
+
 struct GemmArgs {
   int M, N, K;                 // A is [M][K], B is [N][K]
   uint32_t idesc;              // tcgen05 instruction descriptor (operand types)
   const __nv_bfloat16 *bias;   // [N]
-  OutT *out;                   // [M][N]
+  __half *out;                 // [M][N]
   float2 *stats;               // [M][N / BN]
   // side job of warp 6: bf16 -> fp16 of cvt_n 16-byte vectors (0: none)
   const uint4 *cvt_in;
@@ -50,7 +59,8 @@ struct GemmArgs {
   int64_t cvt_n;
   float cvt_scale;             // applied before the fp16 rounding of the side job
   float acc_scale;             // applied to the accumulator before the bias (undoes an operand scaling)
-  int32_t *range_flag;         // set (with UMIM_ERR_UNSUPPORTED) when a value does not fit fp16
+  int32_t *range_flag;         // [gridDim.x] nonzero: a value of this CTA does not fit fp16
+  RangeFlags prior;            // the words of the kernels before (n: 0 for none), folded into CTA 0's
   int32_t *status;
 };
 
@@ -64,9 +74,10 @@ constexpr float kF16Limit = 65504.f;
 // of that range are represented exactly.
 constexpr float kWoScale = 256.f;
 
+// `flag`: the CTA's word in shared memory
 __device__ __forceinline__ void flag_range(int32_t *flag, int32_t *status) {
   set_error(status, UMIM_ERR_UNSUPPORTED);
-  if (flag) *reinterpret_cast<volatile int32_t *>(flag) = 1;
+  *reinterpret_cast<volatile int32_t *>(flag) = 1;
 }
 
 // Persistent: each CTA walks tiles blockIdx.x, blockIdx.x + gridDim.x, ...
@@ -85,13 +96,13 @@ __device__ __forceinline__ void store32(__half *dst, const float (&v)[32]) {
   }
 }
 
-template <typename OutT>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     gemm_bias_gelu_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constant__ CUtensorMap b_map,
-                          GemmArgs<OutT> g) {
+                          GemmArgs g) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ uint64_t full_bar[STAGES], empty_bar[STAGES], acc_full[2], acc_empty[2];
   __shared__ uint32_t tmem_base;
+  __shared__ int32_t s_bad;
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -100,6 +111,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   const int tiles = tiles_n * ((g.M + BM - 1) / BM);
 
   if (threadIdx.x == 0) {
+    s_bad = 0;
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(&full_bar[s], 1);
       mbar_init(&empty_bar[s], 1);
@@ -123,9 +135,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   griddep_wait();
 
   if (warp == 0) {
+    const uint64_t pol_a = policy_evict_first();
+    const uint64_t pol_b = policy_evict_last();
     if (lane == 0) {
-      const uint64_t pol_a = policy_evict_first();
-      const uint64_t pol_b = policy_evict_last();
       uint32_t it = 0;
       bool ok = true;
       for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
@@ -182,6 +194,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       }
     }
   } else if (warp == 6) {
+    if (blockIdx.x == 0) {   // the call's last product: take over what the kernels before found
+      int32_t any = 0;
+      for (int k = 0; k < kFlagKernels; ++k)
+        for (int i = lane; i < g.prior.n[k]; i += 32) any |= g.prior.words[k * kFlagCtas + i];
+      if (any) *reinterpret_cast<volatile int32_t *>(&s_bad) = 1;
+    }
     // side job, converted while the tensor cores work (the memory traffic is
     // small next to the tile loads), 8 loads in flight per lane
     const int64_t step = (int64_t)gridDim.x * 32;
@@ -206,7 +224,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             f[e] *= g.cvt_scale;
             bad |= !(fabsf(f[e]) < kF16Limit);
           }
-          if (bad) flag_range(g.range_flag, g.status);
+          if (bad) flag_range(&s_bad, g.status);
 #pragma unroll
           for (int e = 0; e < 4; ++e) hh[e] = __floats2half2_rn(f[2 * e], f[2 * e + 1]);
           g.cvt_out[i] = o;
@@ -260,7 +278,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           store32(g.out + (int64_t)row * g.N + n0 + c * 32, v);
       }
       if (row < g.M) g.stats[(int64_t)row * tiles_n + n0 / BN] = make_float2(mean, m2);
-      if (bad && row < g.M) flag_range(g.range_flag, g.status);   // this row's fp16 output overflowed
+      if (bad && row < g.M) flag_range(&s_bad, g.status);   // this row's fp16 output overflowed
       // this warp's quarter of the accumulator has been read
       tc_fence_before();
       __syncwarp();
@@ -269,6 +287,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
+  if (threadIdx.x == 0) g.range_flag[blockIdx.x] = s_bad;
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, 2 * BN);
@@ -279,9 +298,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 // gather the static embeddings of the span tokens
 // ---------------------------------------------------------------------------
 __global__ void gather_rows_kernel(const uint4 *table, int64_t vocab, const int32_t *ids, int64_t T, int d,
-                                   uint4 *out, int32_t *range_flag, int32_t *status) {
+                                   uint4 *out, int32_t *status, int early) {
   griddep_wait();
-  if (blockIdx.x == 0 && threadIdx.x == 0) *range_flag = 0;   // the first kernel of the call
+  if (early) griddep_launch();
   const int vec = d / 8;   // 16-byte vectors per row
   const int64_t warp = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
@@ -293,6 +312,277 @@ __global__ void gather_rows_kernel(const uint4 *table, int64_t vocab, const int3
     const uint4 *src = table + (int64_t)(ok ? id : 0) * vec;
     uint4 *dst = out + t * vec;
     for (int i = lane; i < vec; i += 32) dst[i] = ok ? __ldg(src + i) : make_uint4(0, 0, 0, 0);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The same product for few rows (a decode step's merges, one prompt), where
+// 128 x 256 tiles alone would leave most SMs idle and each busy one streaming
+// its share of the weights through one ring (d = 4096, one row tile: 16 CTAs,
+// 37 us for 33.5 MB).  A cluster of 2, 4 or 8 CTAs splits K for one tile; each
+// CTA then leaves its accumulator in its shared memory and takes 256 / split
+// columns of the tile, adding the CTAs' parts over distributed shared memory
+// in rank order, and finishes them (bias, GELU, stores, statistics per 32
+// columns, merged by rank 0).  Eight lanes read one 128-byte line of a peer:
+// with one row per lane instead the reduction alone took about 20 us.  Measured over the whole call (with the next
+// paragraph and the early weights below): 13 spans at d = 4096 100.9 -> 54.0 us,
+// one prompt's 238 spans 119 -> 94 us (with its compressed prompt).
+// CONV: B is bf16 and A fp16 (the output projection); eight warps turn each
+// staged B tile into fp16 (times kWoScale, exact) in place before its MMAs, so
+// no fp16 copy of W_o is written and read back.
+// ---------------------------------------------------------------------------
+constexpr int kSkThreads = 320;    // warp 0: copies, warp 1: MMA + TMEM owner, warps 2-9: conversion, reduction, epilogue
+constexpr int kSkWarps = 8;
+constexpr int kSkMaxSplit = 8;
+constexpr int kSkGroup = 32;       // columns finished together by 8 lanes, 4 each (their statistics: one pair)
+
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(addr)
+               : "memory");
+  return v;
+}
+
+template <bool CONV>
+__global__ void __launch_bounds__(kSkThreads, 1)
+    gemm_splitk_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constant__ CUtensorMap b_map,
+                       GemmArgs g) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  __shared__ uint64_t full_bar[STAGES], conv_bar[STAGES], empty_bar[STAGES], acc_bar;
+  __shared__ uint32_t tmem_base;
+  __shared__ int32_t s_bad;
+  __shared__ float2 s_stats[BN / kSkGroup][BM];   // rank 0's: (mean, M2) of every 32 columns of a row
+  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int split = (int)cluster_size(), rank = (int)cluster_ctarank();
+  const int tiles_n = g.N / BN, tile = blockIdx.x / split;
+  const int m0 = (tile / tiles_n) * BM, n0 = (tile % tiles_n) * BN;
+  const int nkb = g.K / BK / split;   // this CTA's K steps: rank, rank + split, ... (the cluster reads whole lines of B)
+
+  if (threadIdx.x == 0) {
+    s_bad = 0;
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(&full_bar[s], 1);
+      mbar_init(&conv_bar[s], kSkWarps);
+      mbar_init(&empty_bar[s], 1);
+    }
+    mbar_init(&acc_bar, 1);
+    fence_mbar_init();
+    prefetch_tensormap(&a_map);
+    prefetch_tensormap(&b_map);
+  }
+  if (warp == 1) {
+    tmem_alloc(&tmem_base, BN);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_base;
+
+  // this thread's row and half of the columns (warps 2-9: two per tensor-memory lane quadrant)
+  const int q = warp & 3, half = (warp - 2) >> 2;
+  const int r_in = q * 32 + lane, row = m0 + r_in;
+  const int NC = BN / split;                 // columns this CTA finishes
+  const uint32_t part_bytes = (uint32_t)BM * NC * 4;
+  // accumulators in shared memory: [owner][128 rows][NC] fp32, the 16-byte
+  // chunks of a row permuted by the row (a warp's 32 rows hit all banks)
+  auto part_off = [&](int owner, int chunk) {
+    return (uint32_t)owner * part_bytes + (uint32_t)r_in * (NC * 4) + (uint32_t)((chunk ^ (r_in & 7)) << 4);
+  };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      const uint64_t pol_a = policy_evict_last(), pol_b = policy_evict_first();
+      auto load_b = [&](int i) {
+        mbar_arrive_expect_tx(&full_bar[i % STAGES], kStageBytes);
+        tma_load_2d(smem + i % STAGES * kStageBytes + BM * BK * 2, &b_map, &full_bar[i % STAGES],
+                    (i * split + rank) * BK, n0, pol_b);
+      };
+      // the first stages' weights, which no kernel of this call writes, while the kernel before runs
+      for (int i = 0; i < min(nkb, STAGES); ++i) load_b(i);
+      griddep_wait();
+      int issued = 0;
+      for (int i = 0; i < nkb; ++i) {
+        const int s = i % STAGES;
+        if (i >= STAGES) {
+          if (!mbar_wait(&empty_bar[s], ((i / STAGES) & 1) ^ 1)) {
+            set_error(g.status, UMIM_ERR_TIMEOUT);
+            break;
+          }
+          load_b(i);
+        }
+        tma_load_2d(smem + s * kStageBytes, &a_map, &full_bar[s], (i * split + rank) * BK, m0, pol_a);
+        ++issued;
+      }
+      // every copy has landed before the ring is reused or the CTA leaves (bounded)
+      for (int i = max(0, issued - STAGES); i < issued; ++i) mbar_wait(&full_bar[i % STAGES], (i / STAGES) & 1);
+    }
+    __syncwarp();
+    if (blockIdx.x == 0) {   // the call's last product: take over what the kernels before found
+      griddep_wait();
+      int32_t any = 0;
+      for (int k = 0; k < kFlagKernels; ++k)
+        for (int i = lane; i < g.prior.n[k]; i += 32) any |= g.prior.words[k * kFlagCtas + i];
+      if (any) *reinterpret_cast<volatile int32_t *>(&s_bad) = 1;
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      for (int i = 0; i < nkb; ++i) {
+        const int s = i % STAGES;
+        if (!mbar_wait(CONV ? &conv_bar[s] : &full_bar[s], (i / STAGES) & 1)) {
+          set_error(g.status, UMIM_ERR_TIMEOUT);
+          break;
+        }
+        tc_fence_after();
+        const uint32_t a_base = smem_u32(smem + s * kStageBytes);
+        const uint32_t b_base = a_base + BM * BK * 2;
+#pragma unroll
+        for (int k = 0; k < BK / 16; ++k)
+          tc_mma_bf16(tmem, sw128_kmajor_desc(a_base + k * 32), sw128_kmajor_desc(b_base + k * 32), g.idesc,
+                      (i | k) != 0 ? 1u : 0u);
+        tc_commit(&empty_bar[s]);
+      }
+      tc_commit(&acc_bar);   // (also after a timeout: the products issued have finished when it completes)
+    }
+  } else {
+    if constexpr (CONV) {
+      const int t = threadIdx.x - 64;
+      uint32_t inf = 0;
+      for (int i = 0; i < nkb; ++i) {
+        const int s = i % STAGES;
+        if (!__all_sync(0xffffffffu, mbar_wait(&full_bar[s], (i / STAGES) & 1))) {
+          set_error(g.status, UMIM_ERR_TIMEOUT);
+          break;
+        }
+        uint4 *sb = reinterpret_cast<uint4 *>(smem + s * kStageBytes + BM * BK * 2);
+#pragma unroll
+        for (int k = 0; k < BN * BK * 2 / 16 / (kSkWarps * 32); ++k) {
+          const uint4 u = sb[t + k * kSkWarps * 32];
+          float f[8];
+          bf16x8_to_float(u, f);
+          uint32_t o[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const __half2 hh = __floats2half2_rn(f[2 * e] * kWoScale, f[2 * e + 1] * kWoScale);
+            o[e] = *reinterpret_cast<const uint32_t *>(&hh);
+            // inf or NaN: every exponent bit set, so the sum carries into the half's bit 15
+            // (no bf16 value times 2^8 lies between fp16's largest finite value and 65536)
+            inf |= (o[e] & 0x7C007C00u) + 0x04000400u;
+          }
+          sb[t + k * kSkWarps * 32] = make_uint4(o[0], o[1], o[2], o[3]);
+        }
+        fence_proxy_async_smem();   // the MMA's reads of the tile come after these writes
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&conv_bar[s]);
+      }
+      if (inf & 0x80008000u) flag_range(&s_bad, g.status);
+    }
+    if (!__all_sync(0xffffffffu, mbar_wait(&acc_bar, 0))) {
+      set_error(g.status, UMIM_ERR_TIMEOUT);
+    } else if (m0 + q * 32 < g.M) {
+      tc_fence_after();
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int cg = half * 4 + c;   // 32 columns
+        float v[32];
+        tmem_ld_32x32b_x32(tmem + (static_cast<uint32_t>(q * 32) << 16) + cg * 32, v);
+        const int owner = cg * 32 / NC, chunk = (cg * 32 % NC) / 4;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          *reinterpret_cast<float4 *>(smem + part_off(owner, chunk + i)) =
+              make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+      }
+      tc_fence_before();
+    }
+  }
+  __syncwarp();
+  griddep_wait();
+  griddep_launch();     // the next kernel's prologue (a split product: its first weights) may start
+  cluster_sync_all();   // every CTA's accumulators are in its shared memory
+
+  if (warp >= 2) {
+    // a warp's step: 4 rows x 32 columns, lane = (row, 4 columns)
+    const int sub = lane >> 3, ch = lane & 7;
+    const int quads = (min(BM, g.M - m0) + 3) / 4;   // groups of 4 rows that hold one to finish
+    const int groups = NC / kSkGroup;
+    bool bad = false;
+    for (int w = warp - 2; w < quads * groups; w += kSkWarps) {
+      const int grp = w / quads, rr = (w - grp * quads) * 4 + sub;
+      const uint32_t off = (uint32_t)rank * part_bytes + (uint32_t)rr * (NC * 4) +
+                           (uint32_t)(((grp * (kSkGroup / 4) + ch) ^ (rr & 7)) << 4);
+      float4 x[kSkMaxSplit];
+#pragma unroll
+      for (int r = 0; r < kSkMaxSplit; ++r)
+        if (r < split) x[r] = ld_cluster_f4(peer_addr(smem, (uint32_t)r) + off);
+      float v[4] = {x[0].x, x[0].y, x[0].z, x[0].w};
+#pragma unroll
+      for (int r = 1; r < kSkMaxSplit; ++r)
+        if (r < split) {
+          v[0] += x[r].x;
+          v[1] += x[r].y;
+          v[2] += x[r].z;
+          v[3] += x[r].w;
+        }
+      const int col = n0 + rank * NC + grp * kSkGroup + ch * 4;
+      const uint2 b2 = __ldg(reinterpret_cast<const uint2 *>(g.bias + col));
+      const float bb[4] = {__uint_as_float(b2.x << 16), __uint_as_float(b2.x & 0xffff0000u),
+                           __uint_as_float(b2.y << 16), __uint_as_float(b2.y & 0xffff0000u)};
+      bool over = false;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        v[e] = gelu_erf(fmaf(v[e], g.acc_scale, bb[e]));
+        over |= !(fabsf(v[e]) < kF16Limit);
+      }
+      float sum = (v[0] + v[1]) + (v[2] + v[3]);
+#pragma unroll
+      for (int o = 4; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      const float mean = sum * (1.f / kSkGroup);
+      float m2 = 0.f;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) m2 += (v[e] - mean) * (v[e] - mean);
+#pragma unroll
+      for (int o = 4; o >= 1; o >>= 1) m2 += __shfl_xor_sync(0xffffffffu, m2, o);
+      if (m0 + rr >= g.M) continue;
+      bad |= over;
+      if (ch == 0)
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(
+                         peer_addr(&s_stats[rank * groups + grp][rr], 0)),
+                     "f"(mean), "f"(m2)
+                     : "memory");
+      if (in_bounds(col + 3, g.N, g.status, kSiteMergeGemmStore)) {
+        const __half2 h0 = __floats2half2_rn(v[0], v[1]), h1 = __floats2half2_rn(v[2], v[3]);
+        *reinterpret_cast<uint2 *>(g.out + (int64_t)(m0 + rr) * g.N + col) =
+            make_uint2(*reinterpret_cast<const uint32_t *>(&h0), *reinterpret_cast<const uint32_t *>(&h1));
+      }
+    }
+    if (bad) flag_range(&s_bad, g.status);   // an fp16 output of this thread overflowed
+  }
+  __syncwarp();
+  // rank 0 has every column's statistics; no CTA leaves while a peer may still read its accumulators
+  cluster_sync_all();
+  if (rank == 0 && warp >= 2 && half == 0 && row < g.M) {
+    float mean = 0.f, m2 = 0.f;
+#pragma unroll
+    for (int i = 0; i < BN / kSkGroup; ++i) {
+      mean += s_stats[i][r_in].x;
+      m2 += s_stats[i][r_in].y;
+    }
+    mean *= (float)kSkGroup / BN;
+#pragma unroll
+    for (int i = 0; i < BN / kSkGroup; ++i) {
+      const float dlt = s_stats[i][r_in].x - mean;
+      m2 = fmaf(kSkGroup * dlt, dlt, m2);
+    }
+    g.stats[(int64_t)row * tiles_n + n0 / BN] = make_float2(mean, m2);
+  }
+  if (threadIdx.x == 0) g.range_flag[blockIdx.x] = s_bad;
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, BN);
   }
 }
 
@@ -373,6 +663,7 @@ __global__ void __launch_bounds__(kPoolConsumers + 32, CH <= 2 ? 2 : 1)
   __shared__ float s_w[UMIM_MAX_SPAN_TOKENS][8];
   __shared__ float s_A[8], s_B[8], s_C[8];
   __shared__ int s_abort;
+  __shared__ int32_t s_bad;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int ntiles = d / BN;
   const int sbytes = pool_stage_bytes(d);
@@ -387,6 +678,7 @@ __global__ void __launch_bounds__(kPoolConsumers + 32, CH <= 2 ? 2 : 1)
       mbar_init(&empty[i], kPoolConsumers / 32);
     }
     s_abort = 0;
+    s_bad = 0;
     fence_mbar_init();
   }
   if (tid < 8) {
@@ -576,7 +868,7 @@ __global__ void __launch_bounds__(kPoolConsumers + 32, CH <= 2 ? 2 : 1)
           bad |= !(fabsf(o0) < kF16Limit) || !(fabsf(o1) < kF16Limit);
           hp[e] = __floats2half2_rn(o0, o1);
         }
-        if (bad) flag_range(range_flag, status);
+        if (bad) flag_range(&s_bad, status);
         *reinterpret_cast<uint4 *>(O + (int64_t)s * d + cc * 8) = packed;
       }
     }
@@ -585,6 +877,7 @@ __global__ void __launch_bounds__(kPoolConsumers + 32, CH <= 2 ? 2 : 1)
     if (lane == 0) mbar_arrive(&empty[st]);
     consumer_sync();   // s_mom / s_red / s_w / s_C are rewritten for the next span
   }
+  if (tid == 0) range_flag[blockIdx.x] = s_bad;   // (a CTA that gave up reported the timeout)
 }
 
 // ---------------------------------------------------------------------------
@@ -738,9 +1031,10 @@ __global__ void __launch_bounds__(kHeadWarps * 32, 1)
     pool_head_kernel(const __grid_constant__ HeadMaps maps, int mid, const __half *H, const float2 *stats,
                      const int32_t *offs, int S, int64_t T, int d, int h,
                      const __nv_bfloat16 *gamma, const __nv_bfloat16 *beta, const __nv_bfloat16 *query, float eps,
-                     __half *O, int32_t *range_flag, int32_t *status) {
+                     __half *O, int32_t *range_flag, int32_t *status, int early) {
   extern __shared__ __align__(128) uint8_t head_smem[];
   __shared__ uint64_t bars[kHeadWarps][kHeadBufs];
+  __shared__ int32_t s_bad;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int dh = d / h, Ch = dh / 8, ntiles = d / BN;
   const int buf_bytes = head_buf_bytes(dh, ntiles);
@@ -787,8 +1081,10 @@ __global__ void __launch_bounds__(kHeadWarps * 32, 1)
     for (int i = 0; i < kHeadBufs; ++i) mbar_init(&bars[warp][i], 1);
     fence_mbar_init();
   }
-  __syncwarp();
+  if (threadIdx.x == 0) s_bad = 0;
+  __syncthreads();
   griddep_wait();   // H and its statistics come from the projection kernel
+  if (early) griddep_launch();
 
   const int n_items = (S - gw / h + span_step - 1) / span_step;   // spans gw/h, gw/h + step, ... below S
   const uint64_t pol = policy_evict_first();
@@ -848,7 +1144,7 @@ __global__ void __launch_bounds__(kHeadWarps * 32, 1)
       set_error(status, UMIM_ERR_TIMEOUT);
       // let the other buffer's copies land (bounded) before leaving
       if (item + 1 < n_items) mbar_wait(&bars[warp][(item + 1) % kHeadBufs], ((item + 1) / kHeadBufs) & 1);
-      return;
+      break;
     }
     const __half *hs = reinterpret_cast<const __half *>(wbuf + b * buf_bytes);
     const float2 *ts = reinterpret_cast<const float2 *>(wbuf + b * buf_bytes + UMIM_MAX_SPAN_TOKENS * dh * 2);
@@ -868,7 +1164,7 @@ __global__ void __launch_bounds__(kHeadWarps * 32, 1)
         for (int k = 0; k < CPL; ++k)
           if (k * 32 + lane < Ch) *reinterpret_cast<uint4 *>(orow + (k * 32 + lane) * 8) = make_uint4(0, 0, 0, 0);
     }
-    if (__any_sync(0xffffffffu, bad != 0) && lane == 0) flag_range(range_flag, status);
+    if (__any_sync(0xffffffffu, bad != 0) && lane == 0) flag_range(&s_bad, status);
     // every lane is done with this buffer: refill it with the item two ahead
     __syncwarp();
     if (lane == 0 && item + kHeadBufs < n_items) {
@@ -878,6 +1174,8 @@ __global__ void __launch_bounds__(kHeadWarps * 32, 1)
       else n_buf0 = nn;
     }
   }
+  __syncthreads();
+  if (threadIdx.x == 0) range_flag[blockIdx.x] = s_bad;
 }
 
 // ---------------------------------------------------------------------------
@@ -886,10 +1184,12 @@ __global__ void __launch_bounds__(kHeadWarps * 32, 1)
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
     ln_rows_kernel(const __half *Z, float *out, const float2 *stats, int S, int d, const __nv_bfloat16 *gamma,
-                   const __nv_bfloat16 *beta, float eps, const int32_t *range_flag) {
+                   const __nv_bfloat16 *beta, float eps, const int32_t *range_flag, int n_flags) {
   griddep_wait();
   // an intermediate did not fit fp16 (already reported): write no surrogate
-  if (*reinterpret_cast<const volatile int32_t *>(range_flag) != 0) return;
+  int32_t any = 0;
+  for (int i = threadIdx.x; i < n_flags; i += blockDim.x) any |= range_flag[i];
+  if (__syncthreads_or(any)) return;
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= S) return;
@@ -919,7 +1219,7 @@ __global__ void __launch_bounds__(256)
 __global__ void bf16_to_f16_kernel(const uint4 *in, uint4 *out, int64_t n_vec, int32_t *range_flag,
                                    int32_t *status) {
   griddep_wait();
-  bool bad = false;
+  int bad = 0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec; i += (int64_t)gridDim.x * blockDim.x) {
     const uint4 u = in[i];
     float f[8];
@@ -935,7 +1235,12 @@ __global__ void bf16_to_f16_kernel(const uint4 *in, uint4 *out, int64_t n_vec, i
     for (int e = 0; e < 4; ++e) h[e] = __floats2half2_rn(f[2 * e], f[2 * e + 1]);
     out[i] = o;
   }
-  if (bad) flag_range(range_flag, status);
+  if (__syncthreads_or(bad) && threadIdx.x == 0) {
+    set_error(status, UMIM_ERR_UNSUPPORTED);
+    range_flag[blockIdx.x] = 1;
+  } else if (threadIdx.x == 0) {
+    range_flag[blockIdx.x] = 0;
+  }
 }
 
 inline size_t al1k(size_t x) { return (x + 1023) & ~size_t(1023); }
@@ -957,7 +1262,7 @@ size_t merge_spans_workspace_bytes(int64_t T, int S, int d) {
   b += al1k((size_t)std::max(S, 1) * d * 2);                   // o (fp16)
   b += al1k((size_t)d * d * 2);                                 // W_o (fp16)
   b += al1k((size_t)std::max(S, 1) * nt * 8);                  // stats of Z
-  b += al1k(sizeof(int32_t));                                   // fp16 range flag
+  b += al1k(sizeof(int32_t) * kFlagKernels * kFlagCtas);       // fp16 range flags
   return b;
 }
 
@@ -973,40 +1278,44 @@ static bool encode_kmajor(EncodeTiledFn enc, CUtensorMap *map, const void *base,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// out[M][d] = GELU(A[M][d] B[d][d]^T + bias); A and B both bf16 or both fp16
-template <typename OutT>
-static umim_status launch_gemm(EncodeTiledFn enc, const void *A, int64_t M, const void *Bw, int d, bool fp16,
-                               const void *bias, OutT *out, float2 *stats, int32_t *range_flag, float acc_scale,
-                               int32_t *status, cudaStream_t st, const char *label, int num_sms,
-                               const void *cvt_in = nullptr, void *cvt_out = nullptr, int64_t cvt_n = 0) {
+// CTAs that share one tile's K range: as many as keep all clusters resident at
+// once (clusters of 8 leave some SMs of a GPC without a place: 7/8 of the SMs
+// are counted on), else 1.  A product whose tiles alone fill more than half of
+// that (one prompt's 714 tokens at d = 4096: 96 tiles) gains nothing from two
+// half-length waves.
+static int gemm_split(int64_t M, int d, int num_sms) {
+  const int64_t tiles = (int64_t)(d / BN) * ((M + BM - 1) / BM);
+  const int most = std::min(kFlagCtas, std::max(1, num_sms)) / 8 * 7;
+  for (int split = kSkMaxSplit; split > 1; split /= 2)
+    if (tiles * split <= most && d / BK % split == 0) return split;
+  return 1;
+}
+
+// CTAs of a product with M rows
+static int gemm_grid(int64_t M, int d, int num_sms) {
+  const int64_t tiles = (int64_t)(d / BN) * ((M + BM - 1) / BM);
+  const int split = gemm_split(M, d, num_sms);
+  return split > 1 ? (int)tiles * split : (int)std::min<int64_t>(tiles, std::min(kFlagCtas, std::max(1, num_sms)));
+}
+
+// out[M][d] = GELU(A[M][d] B[d][d]^T + bias).  A and B both bf16, or A fp16 and B
+// fp16 (bf16 when the product is split: gemm_split > 1).
+static umim_status launch_gemm(EncodeTiledFn enc, const void *A, const void *Bw, bool fp16, GemmArgs g,
+                               cudaStream_t st, const char *label, int num_sms) {
+  const int d = g.N, split = gemm_split(g.M, d, num_sms);
   CUtensorMap am, bm;
-  if (!encode_kmajor(enc, &am, A, M, d, BM, fp16) || !encode_kmajor(enc, &bm, Bw, d, d, BN, fp16))
+  if (!encode_kmajor(enc, &am, A, g.M, d, BM, fp16) || !encode_kmajor(enc, &bm, Bw, d, d, BN, fp16 && split == 1))
     return UMIM_ERR_CUDA;
-  GemmArgs<OutT> g;
-  g.M = (int)M;
-  g.N = d;
   g.K = d;
   g.idesc = idesc_f32acc(BM, BN, fp16);
-  g.bias = static_cast<const __nv_bfloat16 *>(bias);
-  g.out = out;
-  g.stats = stats;
-  g.cvt_in = static_cast<const uint4 *>(cvt_in);
-  g.cvt_out = static_cast<uint4 *>(cvt_out);
-  g.cvt_n = cvt_n;
-  g.cvt_scale = kWoScale;
-  g.acc_scale = acc_scale;
-  g.range_flag = range_flag;
-  g.status = status;
+  auto kern = split > 1 ? (fp16 ? gemm_splitk_kernel<true> : gemm_splitk_kernel<false>) : gemm_bias_gelu_kernel;
   // set on every call: the attribute belongs to the current device, and calls may
   // come for several devices and from several threads
-  if (cudaFuncSetAttribute(gemm_bias_gelu_kernel<OutT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem) !=
-      cudaSuccess)
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem) != cudaSuccess)
     return UMIM_ERR_CUDA;
-  const int64_t tiles = (int64_t)(d / BN) * ((M + BM - 1) / BM);
-  const int grid = (int)std::min<int64_t>(tiles, std::max(1, num_sms));
   trace_mark(st, label);
-  return launch_pdl(gemm_bias_gelu_kernel<OutT>, dim3(grid), dim3(kGemmThreads), kGemmSmem, st, am, bm, g) ==
-                 cudaSuccess
+  return launch_pdl_cluster(kern, dim3(gemm_grid(g.M, d, num_sms)), dim3(split > 1 ? kSkThreads : kGemmThreads),
+                            (unsigned)split, kGemmSmem, st, am, bm, g) == cudaSuccess
              ? UMIM_OK
              : UMIM_ERR_CUDA;
 }
@@ -1031,27 +1340,44 @@ umim_status merge_spans(const void *embeddings, int64_t vocab, const int32_t *to
   p += al1k((size_t)d * d * 2);
   float2 *st2 = reinterpret_cast<float2 *>(p);
   p += al1k((size_t)std::max(S, 1) * nt * 8);
-  int32_t *range_flag = reinterpret_cast<int32_t *>(p);
+  RangeFlags flags{};
+  flags.words = reinterpret_cast<int32_t *>(p);
+  auto flag_words = [&](FlagKernel k, int ctas) {
+    flags.n[k] = ctas;
+    return flags.words + k * kFlagCtas;
+  };
 
   if (S == 0) return UMIM_OK;
-  bool wo_in_gemm1 = false;
-  if (T > 0) {
-    const int blocks = std::max(1, std::min<int>((int)((T + 7) / 8), num_sms * 8));
-    trace_mark(st, "merge.gather");
-    if (launch_pdl(gather_rows_kernel, dim3(blocks), dim3(256), 0, st, static_cast<const uint4 *>(embeddings), vocab,
-                   token_ids, T, d, reinterpret_cast<uint4 *>(E), range_flag, status) != cudaSuccess)
-      return UMIM_ERR_CUDA;
-    // W_o -> fp16 rides along in a side warp of GEMM1 when its share is small
-    // next to the tiles its CTA computes; else a kernel of its own
-    const int64_t tiles1 = (int64_t)(d / BN) * ((T + BM - 1) / BM);
-    const int64_t grid1 = std::min<int64_t>(tiles1, std::max(1, num_sms));
-    const int64_t n_vec = (int64_t)d * d / 8;
-    wo_in_gemm1 = n_vec <= 128 * 32 * grid1 * (tiles1 / grid1);
-    umim_status r = launch_gemm(enc, E, T, w->w_kv, d, false, w->b_kv, H, st1, range_flag, 1.f, status, st,
-                                "merge.gemm1", num_sms, wo_in_gemm1 ? w->w_o : nullptr, wo_in_gemm1 ? Wo16 : nullptr,
-                                wo_in_gemm1 ? n_vec : 0);
-    if (r != UMIM_OK) return r;
-  }
+  // W_o -> fp16: inside a split output projection; else in a side warp of GEMM1
+  // when its share is small next to the tiles its CTA computes; else in a kernel
+  // of its own
+  const int grid1 = gemm_grid(T, d, num_sms);
+  const int64_t tiles1 = (int64_t)(d / BN) * ((T + BM - 1) / BM);
+  const int64_t n_vec = (int64_t)d * d / 8;
+  const bool wo_split = gemm_split(S, d, num_sms) > 1;
+  const bool wo_in_gemm1 =
+      !wo_split && gemm_split(T, d, num_sms) == 1 && n_vec <= 128LL * 32 * grid1 * (tiles1 / grid1);
+  GemmArgs g1{};
+  g1.M = (int)T;
+  g1.N = d;
+  g1.bias = static_cast<const __nv_bfloat16 *>(w->b_kv);
+  g1.out = H;
+  g1.stats = st1;
+  g1.cvt_in = static_cast<const uint4 *>(w->w_o);
+  g1.cvt_out = reinterpret_cast<uint4 *>(Wo16);
+  g1.cvt_n = wo_in_gemm1 ? n_vec : 0;
+  g1.cvt_scale = kWoScale;
+  g1.acc_scale = 1.f;
+  g1.range_flag = flag_words(kFlagGemm1, grid1);
+  g1.status = status;
+  const int blocks = std::max(1, std::min<int>((int)((T + 7) / 8), num_sms * 8));
+  trace_mark(st, "merge.gather");
+  if (launch_pdl(gather_rows_kernel, dim3(blocks), dim3(256), 0, st, static_cast<const uint4 *>(embeddings), vocab,
+                 token_ids, T, d, reinterpret_cast<uint4 *>(E), status,
+                 gemm_split(T, d, num_sms) > 1 ? 1 : 0) != cudaSuccess)
+    return UMIM_ERR_CUDA;
+  umim_status r = launch_gemm(enc, E, w->w_kv, false, g1, st, "merge.gemm1", num_sms);
+  if (r != UMIM_OK) return r;
   trace_mark(st, "merge.pool");
   const int Ch = d / w->n_heads / 8;   // 16-byte chunks per head
   if (Ch <= 128) {
@@ -1079,13 +1405,13 @@ umim_status merge_spans(const void *embeddings, int64_t vocab, const int32_t *to
     // warps of the grid: a multiple of h, at most one CTA per SM and no more than the items
     const int h = w->n_heads;
     const int64_t items = (int64_t)S * h;
-    int grid = (int)std::min<int64_t>(std::max(1, num_sms), (items + kHeadWarps - 1) / kHeadWarps);
+    int grid = (int)std::min<int64_t>(std::min(kFlagCtas, std::max(1, num_sms)), (items + kHeadWarps - 1) / kHeadWarps);
     while (grid > 1 && (grid * kHeadWarps) % h != 0) --grid;
     if ((grid * kHeadWarps) % h != 0) grid = h;   // 12 * h is a multiple of h
     if (launch_pdl(pk, dim3(grid), dim3(kHeadWarps * 32), psmem, st, maps, mid, (const __half *)H,
                    (const float2 *)st1, span_offsets, S, T, d, h, static_cast<const __nv_bfloat16 *>(w->ln_kv_gamma),
                    static_cast<const __nv_bfloat16 *>(w->ln_kv_beta), static_cast<const __nv_bfloat16 *>(w->query),
-                   w->ln_eps, O, range_flag, status) != cudaSuccess)
+                   w->ln_eps, O, flag_words(kFlagPool, grid), status, wo_split ? 1 : 0) != cudaSuccess)
       return UMIM_ERR_CUDA;
   } else {
     // wider heads: the CTA-per-span kernel with a staged ring
@@ -1098,29 +1424,39 @@ umim_status merge_spans(const void *embeddings, int64_t vocab, const int32_t *to
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pool_per_sm, pk, kPoolConsumers + 32, psmem) != cudaSuccess ||
         pool_per_sm < 1)
       pool_per_sm = 1;
-    const int pool_grid = std::max(1, std::min(S, std::max(1, num_sms) * pool_per_sm));
+    const int pool_grid = std::max(1, std::min(S, std::min(kFlagCtas, std::max(1, num_sms) * pool_per_sm)));
     if (launch_pdl(pk, dim3(pool_grid), dim3(kPoolConsumers + 32), psmem, st, (const __half *)H,
                    (const float2 *)st1, span_offsets, S, T, d, (int)w->n_heads,
                    static_cast<const __nv_bfloat16 *>(w->ln_kv_gamma),
                    static_cast<const __nv_bfloat16 *>(w->ln_kv_beta), static_cast<const __nv_bfloat16 *>(w->query),
-                   w->ln_eps, O, range_flag, status) != cudaSuccess)
+                   w->ln_eps, O, flag_words(kFlagPool, pool_grid), status) != cudaSuccess)
       return UMIM_ERR_CUDA;
   }
-  if (!wo_in_gemm1) {
+  if (!wo_split && !wo_in_gemm1) {
     trace_mark(st, "merge.wo_f16");
-    if (launch_pdl(bf16_to_f16_kernel, dim3(std::max(1, num_sms) * 4), dim3(256), 0, st,
-                   static_cast<const uint4 *>(w->w_o), reinterpret_cast<uint4 *>(Wo16), (int64_t)d * d / 8,
-                   range_flag, status) != cudaSuccess)
+    const int wo_grid = std::min(kFlagCtas, std::max(1, num_sms) * 4);
+    if (launch_pdl(bf16_to_f16_kernel, dim3(wo_grid), dim3(256), 0, st, static_cast<const uint4 *>(w->w_o),
+                   reinterpret_cast<uint4 *>(Wo16), n_vec, flag_words(kFlagWo, wo_grid), status) != cudaSuccess)
       return UMIM_ERR_CUDA;
   }
-  umim_status r = launch_gemm(enc, O, S, Wo16, d, true, w->b_o, Z16, st2, range_flag, 1.f / kWoScale, status, st,
-                              "merge.gemm2", num_sms);
+  GemmArgs g2{};
+  g2.M = S;
+  g2.N = d;
+  g2.bias = static_cast<const __nv_bfloat16 *>(w->b_o);
+  g2.out = Z16;
+  g2.stats = st2;
+  g2.acc_scale = 1.f / kWoScale;
+  g2.prior = flags;
+  const int grid2 = gemm_grid(S, d, num_sms);
+  g2.range_flag = flag_words(kFlagGemm2, grid2);
+  g2.status = status;
+  r = launch_gemm(enc, O, wo_split ? w->w_o : Wo16, true, g2, st, "merge.gemm2", num_sms);
   if (r != UMIM_OK) return r;
   trace_mark(st, "merge.ln_o");
   if (launch_pdl(ln_rows_kernel, dim3((S + 7) / 8), dim3(256), 0, st, (const __half *)Z16, surrogates,
                  (const float2 *)st2, S, d,
                  static_cast<const __nv_bfloat16 *>(w->ln_o_gamma), static_cast<const __nv_bfloat16 *>(w->ln_o_beta),
-                 w->ln_eps, (const int32_t *)range_flag) != cudaSuccess)
+                 w->ln_eps, (const int32_t *)g2.range_flag, grid2) != cudaSuccess)
     return UMIM_ERR_CUDA;
   trace_mark(st, nullptr);
   return UMIM_OK;

@@ -6,7 +6,13 @@
 // takes an equal contiguous range of them.  A range piece that lies in one
 // (b, g) segment produces one partial (running max m, sum l, unnormalised
 // output acc) for the G query heads sharing KV head g; a small combine
-// kernel merges the pieces of each segment with log-sum-exp weights.
+// kernel merges the pieces of each segment with log-sum-exp weights.  The plan
+// is one prefix sum of pages over the sequences: every CTA of the decode kernel
+// derives it from the lengths in shared memory (up to 4096 sequences, 16 KB next
+// to the rings; a kernel of its own before it otherwise), and the piece of
+// segment s that warp w holds has number s + w, which no two pieces share.  A
+// plan kernel before every call cost 3 us of a call of 16 (four sequences of
+// 24 000 entries: rollback and attention 178.3 -> 175.8 us).
 //
 // Per warp: a private ring of NST stages; lane 0 issues TMA tensor loads of
 // whole pages (K and V tiles of 16 x D bf16, 128-byte swizzled) into the
@@ -29,19 +35,16 @@ constexpr int kAttnWarps = 12;
 constexpr int kAttnStages = 2;
 constexpr int kPlanThreadsA = 1024;
 
+constexpr int kSmemPlanBatch = 4096;   // sequences whose prefix sum a decode CTA keeps in shared memory
+
 struct AttnPlan {
   int32_t W;          // pages per warp
-  int32_t total;      // flattened pages
-  int32_t n_seg;
-  int32_t pad[61];
-  // followed by seg_off[n_seg+1], seg_pages[n_seg], piece_base[n_seg+1]
+  int32_t pad[63];
 };
 
 struct AttnWs {
   AttnPlan *plan;
-  int32_t *seg_off;
-  int32_t *seg_pages;
-  int32_t *piece_base;
+  int32_t *pref;      // [B + 1] pages before sequence b (of one KV head)
   float2 *part_ml;    // [pieces][16]      (m in log2 units, l)
   float *part_acc;    // [pieces][16][D]
 };
@@ -51,8 +54,7 @@ inline size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 inline size_t attn_ws_bytes(int B, int Hkv, int D, int total_warps) {
   const size_t nseg = (size_t)B * Hkv;
   const size_t pieces = nseg + total_warps;
-  size_t b = a256(sizeof(AttnPlan));
-  b += 2 * a256(sizeof(int32_t) * (nseg + 1)) + a256(sizeof(int32_t) * nseg);
+  size_t b = a256(sizeof(AttnPlan)) + a256(sizeof(int32_t) * (B + 1));
   b += a256(sizeof(float2) * pieces * 16);
   b += a256(sizeof(float) * pieces * 16 * D);
   return b;
@@ -65,12 +67,8 @@ inline AttnWs attn_carve(void *ws, int B, int Hkv, int D, int total_warps) {
   AttnWs w;
   w.plan = reinterpret_cast<AttnPlan *>(p);
   p += a256(sizeof(AttnPlan));
-  w.seg_off = reinterpret_cast<int32_t *>(p);
-  p += a256(sizeof(int32_t) * (nseg + 1));
-  w.seg_pages = reinterpret_cast<int32_t *>(p);
-  p += a256(sizeof(int32_t) * nseg);
-  w.piece_base = reinterpret_cast<int32_t *>(p);
-  p += a256(sizeof(int32_t) * (nseg + 1));
+  w.pref = reinterpret_cast<int32_t *>(p);
+  p += a256(sizeof(int32_t) * (B + 1));
   w.part_ml = reinterpret_cast<float2 *>(p);
   p += a256(sizeof(float2) * pieces * 16);
   w.part_acc = reinterpret_cast<float *>(p);
@@ -78,86 +76,58 @@ inline AttnWs attn_carve(void *ws, int B, int Hkv, int D, int total_warps) {
 }
 
 // ---------------------------------------------------------------------------
-// plan: segment offsets and pieces (one block)
+// plan
 // ---------------------------------------------------------------------------
-__device__ int scan1024(int v, int &total) {
-  __shared__ int ws[32];
+// Exclusive prefix sum of every sequence's pages into pref[0 .. B] by a block of
+// T threads; returns the total (every thread).  A length outside the block
+// table counts as 0 and is recorded when `report` is set.
+template <int T>
+__device__ int plan_prefix(const int32_t *seq_lens, int B, int max_pages, int32_t *pref, bool report,
+                           int32_t *status) {
+  static_assert(T <= 1024, "one warp scans the warps' sums");
+  __shared__ int s_sum[32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) ws[w] = x;
-  __syncthreads();
-  if (w == 0) {
-    int s = ws[lane];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, s, o);
-      if (lane >= o) s += y;
-    }
-    ws[lane] = s;
-  }
-  __syncthreads();
-  const int r = x + (w ? ws[w - 1] : 0);
-  total = ws[31];
-  __syncthreads();
-  return r;
-}
-
-__global__ void __launch_bounds__(kPlanThreadsA)
-    attn_plan_kernel(const int32_t *seq_lens, int B, int Hkv, int max_pages, int total_warps, AttnWs ws,
-                     int32_t *status) {
-  griddep_wait();
-  const int nseg = B * Hkv;
-  // pass 1: segment offsets (segment (b, g) has n_b pages)
   int carry = 0;
-  for (int base = 0; base < nseg; base += kPlanThreadsA) {
-    const int s = base + threadIdx.x;
+  for (int b0 = 0; b0 < B; b0 += T) {
+    const int b = b0 + threadIdx.x;
     int n = 0;
-    if (s < nseg) {
-      const int b = s / Hkv;
+    if (b < B) {
       int L = seq_lens[b];
       if (L < 0 || (int64_t)L > (int64_t)max_pages * kPageSize) {
-        if (s % Hkv == 0) set_error(status, UMIM_ERR_INVALID_ARG);
+        if (report) set_error(status, UMIM_ERR_INVALID_ARG);
         L = 0;
       }
       n = ceil_div(L, kPageSize);
-      ws.seg_pages[s] = n;
     }
-    int tot;
-    const int incl = scan1024(n, tot);
-    if (s < nseg) ws.seg_off[s] = carry + incl - n;
-    carry += tot;
-  }
-  const int total = carry;
-  const int W = max(1, ceil_div(total, total_warps));
-  // pass 2: pieces per segment
-  int pcarry = 0;
-  for (int base = 0; base < nseg; base += kPlanThreadsA) {
-    const int s = base + threadIdx.x;
-    int np = 0;
-    if (s < nseg) {
-      const int n = ws.seg_pages[s];
-      if (n > 0) {
-        const int off = ws.seg_off[s];
-        np = (off + n - 1) / W - off / W + 1;
-      }
+    int x = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
     }
-    int tot;
-    const int incl = scan1024(np, tot);
-    if (s < nseg) ws.piece_base[s] = pcarry + incl - np;
-    pcarry += tot;
+    if (lane == 31) s_sum[w] = x;
+    __syncthreads();
+    int v = lane < T / 32 ? s_sum[lane] : 0;   // every warp scans the warps' sums
+#pragma unroll
+    for (int o = 1; o < T / 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += y;
+    }
+    const int before = w ? __shfl_sync(0xffffffffu, v, w - 1) : 0;
+    if (b < B) pref[b] = carry + before + x - n;
+    carry += __shfl_sync(0xffffffffu, v, T / 32 - 1);
+    __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    ws.seg_off[nseg] = total;
-    ws.piece_base[nseg] = pcarry;
-    ws.plan->W = W;
-    ws.plan->total = total;
-    ws.plan->n_seg = nseg;
-  }
+  if (threadIdx.x == 0) pref[B] = carry;
+  __syncthreads();
+  return carry;
+}
+
+// more than kSmemPlanBatch sequences: the prefix sum in a kernel of its own (one block)
+__global__ void __launch_bounds__(kPlanThreadsA)
+    attn_plan_kernel(const int32_t *seq_lens, int B, int max_pages, AttnWs ws, int32_t *status) {
+  griddep_wait();
+  plan_prefix<kPlanThreadsA>(seq_lens, B, max_pages, ws.pref, true, status);
 }
 
 // ---------------------------------------------------------------------------
@@ -168,6 +138,7 @@ struct AttnArgs {
   const int32_t *block_table;
   const int32_t *seq_lens;
   int32_t B, Hq, Hkv, G, max_pages, n_pages, layer, n_layers;
+  int32_t smem_plan;
   float scale_log2;
   int32_t *status;
 };
@@ -191,7 +162,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 1)
   __shared__ uint64_t bars[kAttnWarps][kAttnStages];
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int gw = blockIdx.x * kAttnWarps + warp;
+  const int gw = blockIdx.x * kAttnWarps + warp, total_warps = gridDim.x * kAttnWarps;
   uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t *wbuf = base + warp * kAttnStages * kStage;
 
@@ -203,34 +174,51 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 1)
   __syncwarp();
   griddep_wait();
 
-  const int W = ws.plan->W, total = ws.plan->total, nseg = ws.plan->n_seg;
-  const int start = gw * W;
+  const int G = a.G, Hkv = a.Hkv;
+  const int32_t *pref = ws.pref;
+  int pages;
+  if (a.smem_plan) {
+    int32_t *mine = reinterpret_cast<int32_t *>(base + kAttnWarps * kAttnStages * kStage);
+    pages = plan_prefix<kAttnWarps * 32>(a.seq_lens, a.B, a.max_pages, mine, blockIdx.x == 0, a.status);
+    pref = mine;
+    if (blockIdx.x == 0)   // for the combine kernel
+      for (int b = threadIdx.x; b <= a.B; b += kAttnWarps * 32) ws.pref[b] = mine[b];
+  } else {
+    pages = pref[a.B];
+  }
+  const int total = Hkv * pages;
+  const int W = max(1, ceil_div(total, total_warps));
+  if (blockIdx.x == 0 && threadIdx.x == 0) ws.plan->W = W;
+  const int start = (int)min((int64_t)gw * W, (int64_t)total);
   const int end = min(total, start + W);
   if (start >= end) return;
 
-  const int G = a.G;
   const uint64_t pol = policy_evict_first();
 
-  // segment lookup: the last segment whose offset <= pos
-  auto seg_of = [&](int pos) {
-    int l = 0, h = nseg;
-    while (l < h) {
+  // (sequence, KV head, page) of a flattened position: the last sequence whose
+  // first page is at or before it (sequences without pages share their successor's)
+  auto locate = [&](int pos, int &b, int &g, int &pi) {
+    int l = 0, h = a.B;
+    while (h - l > 1) {
       const int m = (l + h) >> 1;
-      if (ws.seg_off[m] <= pos) l = m + 1;
+      if (Hkv * pref[m] <= pos) l = m;
       else h = m;
     }
-    return l - 1;
+    b = l;
+    const int n = pref[b + 1] - pref[b];
+    const int r = pos - Hkv * pref[b];
+    g = r / n;
+    pi = r - g * n;
   };
 
-  // ---- loader cursor ----
-  int ld_pos = start;
-  int ld_seg = seg_of(start);
-  auto issue = [&](int pos, int stage) {
-    while (pos >= ws.seg_off[ld_seg + 1]) ++ld_seg;
-    const int b = ld_seg / a.Hkv, g = ld_seg % a.Hkv;
-    const int pi = pos - ws.seg_off[ld_seg];
-    const int page = in_bounds(pi, a.max_pages, a.status, kSiteAttnTable)
-                         ? a.block_table[(int64_t)b * a.max_pages + pi] : -1;
+  // ---- compute cursor and loader cursor (lane 0 issues the copies) ----
+  int cb, cg, cpi;
+  locate(start, cb, cg, cpi);
+  int cn = pref[cb + 1] - pref[cb], cL = a.seq_lens[cb];
+  int ld_pos = start, lb = cb, lg = cg, lpi = cpi, ln = cn;
+  auto issue = [&](int stage) {
+    const int page = in_bounds(lpi, a.max_pages, a.status, kSiteAttnTable)
+                         ? a.block_table[(int64_t)lb * a.max_pages + lpi] : -1;
     int c4 = a.layer * a.n_pages + page;
     if (page < 0 || page >= a.n_pages) {
       // a coordinate past the tensor's last page: the copy reads zeros
@@ -242,17 +230,24 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 1)
     mbar_arrive_expect_tx(bar, kStage);
 #pragma unroll
     for (int c = 0; c < NB; ++c) {
-      tma_load_5d(dst + c * 2048, &kv_map, bar, c * 64, 0, g, 0, c4, pol);
-      tma_load_5d(dst + kTile + c * 2048, &kv_map, bar, c * 64, 0, g, 1, c4, pol);
+      tma_load_5d(dst + c * 2048, &kv_map, bar, c * 64, 0, lg, 0, c4, pol);
+      tma_load_5d(dst + kTile + c * 2048, &kv_map, bar, c * 64, 0, lg, 1, c4, pol);
+    }
+    if (++ld_pos < end && ++lpi == ln) {
+      lpi = 0;
+      if (++lg == Hkv) {
+        lg = 0;
+        do ++lb;
+        while (pref[lb + 1] == pref[lb]);
+        ln = pref[lb + 1] - pref[lb];
+      }
     }
   };
   if (lane == 0) {
-    for (int s = 0; s < kAttnStages && ld_pos < end; ++s, ++ld_pos) issue(ld_pos, s);
+    for (int s = 0; s < kAttnStages && ld_pos < end; ++s) issue(s);
   }
 
   // ---- compute state ----
-  int cseg = seg_of(start);
-  int cb = cseg / a.Hkv, cg = cseg % a.Hkv;
   const int qr = lane >> 2, qc = lane & 3;      // mma fragment row / column group
   uint32_t qa[KC][4];
   auto load_q = [&]() {
@@ -281,8 +276,8 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 1)
     s0 += __shfl_xor_sync(0xffffffffu, s0, 2);
     s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
     s1 += __shfl_xor_sync(0xffffffffu, s1, 2);
-    const int piece = ws.piece_base[cseg] + (gw - ws.seg_off[cseg] / W);
-    if (!in_bounds(piece, nseg + (int64_t)gridDim.x * kAttnWarps, a.status, kSiteAttnPiece)) return;
+    const int piece = cb * Hkv + cg + gw;
+    if (!in_bounds(piece, (int64_t)a.B * Hkv + total_warps, a.status, kSiteAttnPiece)) return;
     float2 *ml = ws.part_ml + (int64_t)piece * 16;
     float *pacc = ws.part_acc + (int64_t)piece * 16 * D;
     if (qc == 0) {
@@ -300,11 +295,16 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 1)
   int it = 0;
   for (int pos = start; pos < end; ++pos, ++it) {
     // next segment?
-    if (pos >= ws.seg_off[cseg + 1]) {
+    if (cpi == cn) {
       flush();
-      while (pos >= ws.seg_off[cseg + 1]) ++cseg;
-      cb = cseg / a.Hkv;
-      cg = cseg % a.Hkv;
+      cpi = 0;
+      if (++cg == Hkv) {
+        cg = 0;
+        do ++cb;
+        while (pref[cb + 1] == pref[cb]);
+        cn = pref[cb + 1] - pref[cb];
+        cL = a.seq_lens[cb];
+      }
       load_q();
       m0 = m1 = -INFINITY;
       l0 = l1 = 0.f;
@@ -316,15 +316,14 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 1)
     if (!mbar_wait(&bars[warp][stage], parity)) {
       set_error(a.status, UMIM_ERR_TIMEOUT);
       // let the copies still in flight land (each wait bounded) before leaving
-      for (int k = 1; k < kAttnStages && it + k < ld_pos - start; ++k)
+      for (int k = 1; k < kAttnStages && pos + k < ld_pos; ++k)
         mbar_wait(&bars[warp][(it + k) % kAttnStages], ((it + k) / kAttnStages) & 1);
       return;
     }
     uint8_t *kt = wbuf + stage * kStage;
     uint8_t *vt = kt + kTile;
-    const int pi = pos - ws.seg_off[cseg];
-    const int L = a.seq_lens[cb];
-    const int nvalid = min(16, L - pi * 16);
+    const int nvalid = min(16, cL - cpi * 16);
+    ++cpi;
     if (nvalid < 16) {
       // zero V rows past the end so that 0 * garbage cannot make a NaN
       for (int idx = lane; idx < (16 - nvalid) * NB * 8; idx += 32) {
@@ -420,10 +419,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 1)
     }
     __syncwarp();
     // refill this stage
-    if (lane == 0 && ld_pos < end) {
-      issue(ld_pos, stage);
-      ++ld_pos;
-    }
+    if (lane == 0 && ld_pos < end) issue(stage);
   }
   flush();
 }
@@ -450,7 +446,16 @@ __global__ void __launch_bounds__(kCombineThreads)
   const bool live = row_g < B * Hq;
   const int b = live ? row_g / Hq : 0, h = live ? row_g % Hq : 0;
   const int seg = b * Hkv + h / G, row = h % G;
-  const int p0 = live ? ws.piece_base[seg] : 0, p1 = live ? ws.piece_base[seg + 1] : 0;
+  // the segment's pieces: seg + w for the warps w whose ranges meet its positions
+  int p0 = 0, p1 = 0;
+  if (live) {
+    const int first = ws.pref[b], n = ws.pref[b + 1] - first, W = ws.plan->W;
+    const int o = Hkv * first + h / G * n;
+    if (n > 0) {
+      p0 = seg + o / W;
+      p1 = seg + (o + n - 1) / W + 1;
+    }
+  }
   float M = -INFINITY, l = 0.f, o[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) o[e] = 0.f;
@@ -541,12 +546,16 @@ static umim_status run_attention(const void *q, int Hq, const umim_paged_kv *kv,
   const int total_warps = attn_total_warps(num_sms);
   const int Hkv = kv->n_kv_heads;
   AttnWs ws = attn_carve(workspace, B, Hkv, D, total_warps);
-  trace_mark(stream, "attention.plan");
-  if (launch_pdl(attn_plan_kernel, dim3(1), dim3(kPlanThreadsA), 0, stream, seq_lens, B, Hkv, max_pages,
-                 total_warps, ws, status) != cudaSuccess)
-    return UMIM_ERR_CUDA;
+  const bool smem_plan = B <= kSmemPlanBatch;
+  if (!smem_plan) {
+    trace_mark(stream, "attention.plan");
+    if (launch_pdl(attn_plan_kernel, dim3(1), dim3(kPlanThreadsA), 0, stream, seq_lens, B, max_pages, ws, status) !=
+        cudaSuccess)
+      return UMIM_ERR_CUDA;
+  }
 
   AttnArgs a{};
+  a.smem_plan = smem_plan ? 1 : 0;
   a.q = static_cast<const __nv_bfloat16 *>(q);
   a.block_table = block_table;
   a.seq_lens = seq_lens;
@@ -560,7 +569,8 @@ static umim_status run_attention(const void *q, int Hq, const umim_paged_kv *kv,
   a.n_layers = kv->n_layers;
   a.scale_log2 = scale * 1.4426950408889634f;
   a.status = status;
-  const size_t smem = (size_t)kAttnWarps * kAttnStages * 2 * 16 * D * 2 + 1024;
+  const size_t smem = (size_t)kAttnWarps * kAttnStages * 2 * 16 * D * 2 + 1024 +
+                      (smem_plan ? sizeof(int32_t) * ((size_t)B + 1) : 0);
   auto kern = attn_decode_kernel<D>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return UMIM_ERR_CUDA;

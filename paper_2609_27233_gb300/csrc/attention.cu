@@ -459,18 +459,45 @@ __global__ void __launch_bounds__(kCombineThreads)
   float M = -INFINITY, l = 0.f, o[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) o[e] = 0.f;
-  for (int pc = p0 + sub; pc < p1; pc += WPR) {
-    const float2 ml = ws.part_ml[(int64_t)pc * 16 + row];
-    const float *acc = ws.part_acc + ((int64_t)pc * 16 + row) * D + lane * E;
-    float av[E];
+  // pieces whose loads are in flight together: one at a time, a row of 76 pieces
+  // (long context, 16.4 us with eight warps a row) waits for memory ten times over;
+  // four at a time 8.3 us
+  constexpr int U = 4;
+  for (int pc = p0 + sub; pc < p1; pc += U * WPR) {
+    float2 ml[U];
+    float av[U][E];
 #pragma unroll
-    for (int e = 0; e < E; ++e) av[e] = acc[e];
-    const float nm = fmaxf(M, ml.x);
+    for (int u = 0; u < U; ++u) {
+      const int64_t at = (int64_t)(pc + u * WPR) * 16 + row;
+      ml[u] = make_float2(-INFINITY, 0.f);
+#pragma unroll
+      for (int e = 0; e < E; ++e) av[u][e] = 0.f;
+      if (pc + u * WPR < p1) {
+        ml[u] = ws.part_ml[at];
+        if constexpr (E == 4) {
+          const float4 f = *reinterpret_cast<const float4 *>(ws.part_acc + at * D + lane * E);
+          av[u][0] = f.x, av[u][1] = f.y, av[u][2] = f.z, av[u][3] = f.w;
+        } else {
+          const float2 f = *reinterpret_cast<const float2 *>(ws.part_acc + at * D + lane * E);
+          av[u][0] = f.x, av[u][1] = f.y;
+        }
+      }
+    }
+    float nm = M;
+#pragma unroll
+    for (int u = 0; u < U; ++u) nm = fmaxf(nm, ml[u].x);
     if (nm == -INFINITY) continue;   // nothing but empty pieces so far
-    const float c_old = exp2f(M - nm), c_new = exp2f(ml.x - nm);
-    l = l * c_old + ml.y * c_new;
+    const float c_old = exp2f(M - nm);
+    l *= c_old;
 #pragma unroll
-    for (int e = 0; e < E; ++e) o[e] = o[e] * c_old + av[e] * c_new;
+    for (int e = 0; e < E; ++e) o[e] *= c_old;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const float c = exp2f(ml[u].x - nm);   // 0 for an absent or empty piece
+      l = fmaf(ml[u].y, c, l);
+#pragma unroll
+      for (int e = 0; e < E; ++e) o[e] = fmaf(av[u][e], c, o[e]);
+    }
     M = nm;
   }
   if constexpr (WPR > 1) {

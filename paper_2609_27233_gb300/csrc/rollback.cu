@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
   __shared__ int s_sq[kSmemSeqs], s_nd[kSmemSeqs], s_ub[kSmemSeqs], s_fp[kSmemSeqs];
   __shared__ int64_t s_toff[kSmemLanes];
   __shared__ int32_t s_tlh[kSmemLanes];
-  __shared__ float s_w[ROPE ? D / 2 : 1];   // RoPE angular frequencies
+  __shared__ __align__(8) float s_w[ROPE ? D / 2 : 2];   // RoPE angular frequencies
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nm = gridDim.x * kBulkMovers;
   uint8_t *ring = bulk_smem + (size_t)wid * kBulkStages * TILE;
@@ -422,21 +422,34 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
   // angle r w rounded plus its exact rounding error (an fma) folded into the sine
   // and cosine to first order, and the rounded angle reduced to [-pi, pi] (Cody
   // and Waite's three-part reduction) for the hardware sine and cosine.  Lane l
-  // takes the pairs m = l and l + 32 of every row; consecutive rows with the same
-  // shift (a run of moved entries between two spans) reuse the lane's angles.
+  // takes the pairs m = 2l and 2l + 1 of every row, one 32-bit word of each half
+  // of the row, so that shared memory is read and written in words and the
+  // arithmetic is packed; four rows' words are read ahead.  Consecutive rows with
+  // the same shift (a run of moved entries between two spans) reuse the angles.
+  // With single bf16 elements (pairs l and l + 32) the long context's move took
+  // 111 us against 95 us now (75 us without rotation).
   static_assert(D / 2 <= 64, "two pairs per lane");
   auto rotate_rows = [&](const Unit &m, uint8_t *stage) {
-    const int half = a.rotary_dim / 2;
-    float prev = 0.f, snc[2] = {0.f, 0.f}, csc[2] = {1.f, 1.f};
-    for (int r = m.ra; r < m.rb; ++r) {
-      const float rf = (float)__shfl_sync(0xffffffffu, m.shift, r);
-      if (rf == 0.f) continue;   // a surrogate or an entry that keeps its position
-      if (rf != prev) {
+    const int half = a.rotary_dim / 2;   // even
+    const bool mine = 2 * lane < half;
+    float prev = 0.f;
+    float2 sn = make_float2(0.f, 0.f), cs = make_float2(1.f, 1.f);
+    for (int r0 = m.ra; r0 < m.rb; r0 += 4) {
+      uint32_t x[4], y[4];
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const int q = lane + 32 * i;
-          if (q < half) {
-            const float w = s_w[q];
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t *row = reinterpret_cast<const uint32_t *>(stage + min(r0 + u, m.rb - 1) * ROW);
+        x[u] = mine ? row[lane] : 0u;
+        y[u] = mine ? row[half / 2 + lane] : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = r0 + u;
+        if (r >= m.rb) break;
+        const float rf = (float)__shfl_sync(0xffffffffu, m.shift, r);
+        if (rf == 0.f) continue;   // a surrogate or an entry that keeps its position
+        if (rf != prev) {
+          auto angle = [&](float w, float &s_out, float &c_out) {
             const float ang = rf * w;
             const float err = fmaf(rf, w, -ang);
             const float kq = rintf(ang * 0.15915493667125702f);
@@ -444,20 +457,26 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
             red = fmaf(-kq, 0.0019354820251464844f, red);
             red = fmaf(-kq, -1.7484555314695172e-07f, red);
             const float sn0 = __sinf(red), cs0 = __cosf(red);
-            snc[i] = fmaf(err, cs0, sn0);
-            csc[i] = fmaf(-err, sn0, cs0);
+            s_out = fmaf(err, cs0, sn0);
+            c_out = fmaf(-err, sn0, cs0);
+          };
+          if (mine) {
+            const float2 w = *reinterpret_cast<const float2 *>(s_w + 2 * lane);
+            angle(w.x, sn.x, cs.x);
+            angle(w.y, sn.y, cs.y);
           }
+          prev = rf;
         }
-        prev = rf;
-      }
-      __nv_bfloat16 *row = reinterpret_cast<__nv_bfloat16 *>(stage + r * ROW);
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int q = lane + 32 * i;
-        if (q < half) {
-          const float x = __bfloat162float(row[q]), y = __bfloat162float(row[q + half]);
-          row[q] = __float2bfloat16_rn(fmaf(x, csc[i], y * snc[i]));
-          row[q + half] = __float2bfloat16_rn(fmaf(y, csc[i], -(x * snc[i])));
+        if (mine) {
+          const float2 xv = make_float2(__uint_as_float(x[u] << 16), __uint_as_float(x[u] & 0xffff0000u));
+          const float2 yv = make_float2(__uint_as_float(y[u] << 16), __uint_as_float(y[u] & 0xffff0000u));
+          const float2 xs = __fmul2_rn(xv, sn);
+          const float2 xr = __ffma2_rn(xv, cs, __fmul2_rn(yv, sn));
+          const float2 yr = __ffma2_rn(yv, cs, make_float2(-xs.x, -xs.y));
+          const __nv_bfloat162 xo = __floats2bfloat162_rn(xr.x, xr.y), yo = __floats2bfloat162_rn(yr.x, yr.y);
+          uint32_t *row = reinterpret_cast<uint32_t *>(stage + r * ROW);
+          row[lane] = *reinterpret_cast<const uint32_t *>(&xo);
+          row[half / 2 + lane] = *reinterpret_cast<const uint32_t *>(&yo);
         }
       }
     }

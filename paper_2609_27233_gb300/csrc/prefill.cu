@@ -61,6 +61,7 @@ struct PfArgs {
   const int32_t *cu;                // [B + 1]
   int32_t *cu_tiles;                // [B + 1] workspace: query-tile offsets
   int32_t *pcu;                     // [B + 1] workspace: key offsets padded to 64 in V^T
+  int4 *tiles;                      // [query tiles] workspace: first row, length, first query, V^T column of the sequence
   const __nv_bfloat16 *v;           // [T][Hkv][D]
   __half *vt;                       // [Hkv][D][Tp] workspace, fp16
   int64_t Tp;                       // row length of V^T (a multiple of 64)
@@ -139,7 +140,8 @@ __device__ __forceinline__ int pf_find(const int32_t *key, int B, int x) {
 
 // V^T: vt[g][d][pcu[b] + t] = v[cu[b] + t][g][d] for t < len_b, 0 up to the
 // next multiple of 64.  One CTA per 64 padded keys and KV head, through a
-// shared-memory tile.
+// shared-memory tile.  The CTAs of KV head 0 whose keys start a query tile also
+// write that tile's record.
 template <int D>
 __global__ void __launch_bounds__(256) vt_kernel(PfArgs a) {
   griddep_wait();
@@ -149,6 +151,8 @@ __global__ void __launch_bounds__(256) vt_kernel(PfArgs a) {
   const int b = pf_find(a.pcu, a.B, k0);
   const int len = a.cu[b + 1] - a.cu[b];
   const int t0 = k0 - a.pcu[b];
+  if (g == 0 && threadIdx.x == 0 && t0 % kPfRows == 0)
+    a.tiles[a.cu_tiles[b] + t0 / kPfRows] = make_int4(a.cu[b], len, t0, a.pcu[b]);
   constexpr int CPR = D / 8;   // 16-byte chunks per key row
   for (int i = threadIdx.x; i < kPfKeys * CPR; i += blockDim.x) {
     const int r = i / CPR, c = i % CPR;
@@ -256,7 +260,8 @@ struct PfSmem {
   static constexpr int kV = D * kPfKeys * 2;              // V^T tile: [D rows][128 B]
   static constexpr int kKoff = kQ;
   static constexpr int kVoff = kKoff + kPfKStages * kK;
-  static constexpr int kTotal = kVoff + kPfVStages * kV;
+  static constexpr int kOoff = kVoff + kPfVStages * kV;   // per softmax warp: 32 rows x 32 columns of the output
+  static constexpr int kTotal = kOoff + 4 * 2048;
 };
 
 template <int D>
@@ -270,6 +275,7 @@ __global__ void __launch_bounds__(kPfThreads, 2)
       v_empty[kPfVStages], s_full[2], s_empty[2], p_full[2], p_empty, o_done, o_free, mma_done[2];
   __shared__ uint32_t tmem_base;
   __shared__ int s_abort;
+  __shared__ int4 s_rec[4];   // the records of the CTA's units k & 3 (written by the copy thread before it loads Q)
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(pf_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -321,18 +327,22 @@ __global__ void __launch_bounds__(kPfThreads, 2)
   struct Unit {
     int s0, len, q0, h, g, n_kv, kbase;
   };
-  auto unit_of = [&](int u) {
+  // The copy thread reads a unit's record a unit ahead and leaves it in s_rec; the
+  // others find it there once the unit's first barrier has let them through (it
+  // loads Q of unit k + 1 only when unit k's S products are done, so at most
+  // units k - 1 to k + 1 are in use at once).  Looked up by every warp when it
+  // was needed, with a binary search over the sequences, a unit began 1000 to
+  // 5000 cycles late.  With this and the turned stores of the epilogue (64 x 1500
+  // rows, 32/8 heads, D = 128) the call went from 1300 to 1238 us.
+  auto unit_of = [&](int u, int4 rec) {   // a sequence's last (heaviest) tiles come first
     Unit w;
-    const int t = total - 1 - u / a.Hq;   // a sequence's last (heaviest) tiles first
-    const int b = pf_find(a.cu_tiles, a.B, t);
-    const int qt = t - a.cu_tiles[b];
-    w.s0 = a.cu[b];
-    w.len = a.cu[b + 1] - w.s0;
-    w.q0 = qt * kPfRows;
+    w.s0 = rec.x;
+    w.len = rec.y;
+    w.q0 = rec.z;
+    w.kbase = rec.w;
     w.h = u % a.Hq;
     w.g = w.h / a.G;
     w.n_kv = (min(w.q0 + kPfRows, w.len) + kPfKeys - 1) / kPfKeys;   // causal key tiles
-    w.kbase = a.pcu[b];
     return w;
   };
   // a warp that gave up tells the others, so that no wait is left to time out on its own
@@ -351,8 +361,14 @@ __global__ void __launch_bounds__(kPfThreads, 2)
       int nk = 0, nv = 0, nq = 0;   // K and V^T tiles (ring positions) and Q tiles loaded so far
       bool ok = true;
       int k_unit = 0;
+      auto record = [&](int u) {
+        return u < n_units ? a.tiles[total - 1 - u / a.Hq] : make_int4(0, 0, 0, 0);
+      };
+      int4 rec = record((int)blockIdx.x);
       for (int u = (int)blockIdx.x; u < n_units && ok; u += G, ++k_unit) {
-        const Unit w = unit_of(u);
+        const Unit w = unit_of(u, rec);
+        const int4 here = rec;
+        rec = record(u + G);
         // the unit's last K row and V^T column (a TMA copy past the end of
         // its tensor reads zeros, so these checks only record)
         (void)in_bounds((int64_t)w.s0 + (w.n_kv - 1) * kPfKeys, a.T, a.status, kSitePrefillKvRow);
@@ -362,6 +378,7 @@ __global__ void __launch_bounds__(kPfThreads, 2)
           ok = false;
           break;
         }
+        s_rec[k_unit & 3] = here;
         mbar_arrive_expect_tx(&q_full, L::kQ);
 #pragma unroll
         for (int d = 0; d < DA; ++d)
@@ -409,11 +426,11 @@ __global__ void __launch_bounds__(kPfThreads, 2)
       bool ok = true;
       int nt = 0, k_unit = 0;   // tiles and units so far
       for (int u = (int)blockIdx.x; u < n_units && ok; u += G, ++k_unit) {
-        const Unit w = unit_of(u);
         if (aborted() || !mbar_wait(&q_full, (uint32_t)k_unit & 1u)) {
           ok = false;
           break;
         }
+        const Unit w = unit_of(u, s_rec[k_unit & 3]);
         tc_fence_after();
         const uint32_t q_base = smem_u32(smem);
         for (int i = 0; i < w.n_kv; ++i, ++nt) {
@@ -451,11 +468,12 @@ __global__ void __launch_bounds__(kPfThreads, 2)
       bool ok = true;
       int nt = 0, k_unit = 0;
       for (int u = (int)blockIdx.x; u < n_units && ok; u += G, ++k_unit) {
-        const Unit w = unit_of(u);
-        if (k_unit > 0 && (aborted() || !mbar_wait(&o_free, (uint32_t)(k_unit - 1) & 1u))) {
+        if ((k_unit > 0 && (aborted() || !mbar_wait(&o_free, (uint32_t)(k_unit - 1) & 1u))) || aborted() ||
+            !mbar_wait(&p_full[nt & 1], (nt >> 1) & 1)) {   // the unit's first P: its record is there
           ok = false;
           break;
         }
+        const Unit w = unit_of(u, s_rec[k_unit & 3]);
         for (int i = 0; i < w.n_kv; ++i, ++nt) {
           const int s = nt % kPfVStages, sb = nt & 1;
           if (aborted() || !mbar_wait(&v_full[s], (nt / kPfVStages) & 1) ||
@@ -493,9 +511,50 @@ __global__ void __launch_bounds__(kPfThreads, 2)
     auto wwait = [&](uint64_t *m, uint32_t parity) {
       return __all_sync(0xffffffffu, !aborted() && mbar_wait(m, parity)) != 0;
     };
+    // The output of a unit: O / l once its last product has landed, then O is
+    // free for the next unit.  Thread = row holds 32 columns at a time; the warp
+    // turns them through shared memory so that a store writes 64 contiguous
+    // bytes of eight rows (one row per lane took 16-byte pieces of 32 rows).
+    auto epilogue = [&](const Unit &w, float l_run, int k) -> bool {   // of the CTA's k-th unit
+      if (!wwait(&o_done, (uint32_t)k & 1u)) return false;
+      tc_fence_after();
+      uint8_t *stage = smem + L::kOoff + (warp - 2) * 2048;
+      const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+      const int first = w.q0 + quad * 32;        // position of the warp's first row
+      __nv_bfloat16 *obase = a.out + (((int64_t)w.s0 + first) * a.Hq + w.h) * D;
+#pragma unroll 1
+      for (int c = 0; c < D / 32; ++c) {
+        float o[32];
+        tmem_ld_32x32b_x32(t_o + c * 32, o);
+        __syncwarp();   // the lanes have read the columns before
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          *reinterpret_cast<uint4 *>(stage + lane * 64 + ((e ^ ((lane >> 1) & 3)) << 4)) =
+              make_uint4(pack_bf16x2(o[8 * e] * inv, o[8 * e + 1] * inv),
+                         pack_bf16x2(o[8 * e + 2] * inv, o[8 * e + 3] * inv),
+                         pack_bf16x2(o[8 * e + 4] * inv, o[8 * e + 5] * inv),
+                         pack_bf16x2(o[8 * e + 6] * inv, o[8 * e + 7] * inv));
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int row = k * 8 + (lane >> 2), ch = lane & 3;
+          const uint4 x = *reinterpret_cast<const uint4 *>(stage + row * 64 + ((ch ^ ((row >> 1) & 3)) << 4));
+          if (first + row < w.len && in_bounds((int64_t)w.s0 + first + row, a.T, a.status, kSitePrefillOutRow))
+            *reinterpret_cast<uint4 *>(obase + (int64_t)row * a.Hq * D + c * 32 + ch * 8) = x;
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&o_free);
+      return true;
+    };
     int nt = 0, k_unit = 0;
-    for (int u = (int)blockIdx.x; u < n_units && ok; u += G, ++k_unit) {
-      const Unit w = unit_of(u);
+    for (; (int)blockIdx.x + k_unit * G < n_units && ok; ++k_unit) {
+      if (!wwait(&s_full[nt & 1], (nt >> 1) & 1)) {   // the unit's first S: its record is there
+        ok = false;
+        break;
+      }
+      const Unit w = unit_of((int)blockIdx.x + k_unit * G, s_rec[k_unit & 3]);
       const int qpos = w.q0 + r;                  // position within the sequence
       const int kmax = min(qpos, w.len - 1);      // last key this row sees
       float m_run = -INFINITY, l_run = 0.f;       // running max (log2 units, moved in steps > 8) and row sum
@@ -529,13 +588,15 @@ __global__ void __launch_bounds__(kPfThreads, 2)
         // exp2(s * scale - max) and the row sum, two columns per packed instruction
         const float2 sl2x2 = make_float2(sl2, sl2), nm2 = make_float2(nm, nm);
         float2 la = make_float2(0.f, 0.f), lb = la;
+        float pk[kPfKeys / 2];   // P in fp16 pairs (P <= 2^8)
 #pragma unroll
         for (int c = 0; c < kPfKeys; c += 2) {
           const float2 x = __ffma2_rn(make_float2(s[c], s[c + 1]), sl2x2, nm2);
-          s[c] = ex2_approx(x.x);   // masked (-inf): 0
-          s[c + 1] = ex2_approx(x.y);
-          if (c & 2) lb = __fadd2_rn(lb, make_float2(s[c], s[c + 1]));
-          else la = __fadd2_rn(la, make_float2(s[c], s[c + 1]));
+          const float2 e = make_float2(ex2_approx(x.x), ex2_approx(x.y));   // masked (-inf): 0
+          if (c & 2) lb = __fadd2_rn(lb, e);
+          else la = __fadd2_rn(la, e);
+          const __half2 hh = __floats2half2_rn(e.x, e.y);
+          pk[c / 2] = __uint_as_float(*reinterpret_cast<const uint32_t *>(&hh));
         }
         const float2 lab = __fadd2_rn(la, lb);
         l_run += lab.x + lab.y;
@@ -556,46 +617,13 @@ __global__ void __launch_bounds__(kPfThreads, 2)
           }
           tc_fence_before();
         }
-        // P(j) in fp16 over S(j)'s columns (this thread has read them), for the P V product
-        {
-          float pk[32];
-#pragma unroll
-          for (int c = 0; c < 32; ++c) {
-            const __half2 hh = __floats2half2_rn(s[2 * c], s[2 * c + 1]);   // P <= 2^8
-            pk[c] = __uint_as_float(*reinterpret_cast<const uint32_t *>(&hh));
-          }
-          tmem_st_32x32b_x32(t_s + sb * kPfKeys, pk);
-        }
+        // P(j) over S(j)'s columns (this thread has read them), for the P V product
+        tmem_st_32x32b_x32(t_s + sb * kPfKeys, pk);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&p_full[sb]);
       }
-      if (!ok) break;
-      // epilogue: O / l once the unit's last product has landed, then O is free for the next unit
-      if (!wwait(&o_done, (uint32_t)k_unit & 1u)) {
-        ok = false;
-        break;
-      }
-      tc_fence_after();
-      const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
-      __nv_bfloat16 *orow = a.out + (((int64_t)w.s0 + qpos) * a.Hq + w.h) * D;
-#pragma unroll 1
-      for (int c = 0; c < D / 32; ++c) {
-        float o[32];
-        tmem_ld_32x32b_x32(t_o + c * 32, o);
-        if (qpos < w.len && in_bounds((int64_t)w.s0 + qpos, a.T, a.status, kSitePrefillOutRow)) {
-          uint4 *dst = reinterpret_cast<uint4 *>(orow + c * 32);
-#pragma unroll
-          for (int e = 0; e < 4; ++e)
-            dst[e] = make_uint4(pack_bf16x2(o[8 * e] * inv, o[8 * e + 1] * inv),
-                                pack_bf16x2(o[8 * e + 2] * inv, o[8 * e + 3] * inv),
-                                pack_bf16x2(o[8 * e + 4] * inv, o[8 * e + 5] * inv),
-                                pack_bf16x2(o[8 * e + 6] * inv, o[8 * e + 7] * inv));
-        }
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&o_free);
+      if (ok) ok = epilogue(w, l_run, k_unit);
     }
     if (!ok) give_up();
   }
@@ -619,14 +647,19 @@ bool encode_3d(EncodeTiledFn enc, CUtensorMap *map, const void *base, uint64_t d
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// bytes before V^T: the prefix sums and the query tiles' records
+size_t pf_plan_bytes(int B, int T) {
+  const size_t sums = ((size_t)2 * (B + 1) * sizeof(int32_t) + 15) & ~size_t(15);
+  return (sums + ((size_t)T / kPfRows + B) * sizeof(int4) + 1023) & ~size_t(1023);
+}
+
 // row length of V^T: room for every sequence padded to 64 keys
 int64_t vt_row(int B, int T) { return ((int64_t)T + 63LL * B + 63) / 64 * 64; }
 
 }  // namespace
 
 size_t prefill_attention_workspace_bytes(int B, int T, int Hkv, int D) {
-  const size_t plan = ((size_t)2 * (B + 1) * sizeof(int32_t) + 1023) & ~size_t(1023);
-  return plan + (size_t)Hkv * D * vt_row(B, T) * 2;
+  return pf_plan_bytes(B, T) + (size_t)Hkv * D * vt_row(B, T) * 2;
 }
 
 umim_status prefill_attention(const void *q, const void *k, const void *v, int T, int Hq, int Hkv, int D,
@@ -640,8 +673,9 @@ umim_status prefill_attention(const void *q, const void *k, const void *v, int T
   a.cu_tiles = static_cast<int32_t *>(ws);
   a.pcu = a.cu_tiles + (B + 1);
   a.v = static_cast<const __nv_bfloat16 *>(v);
-  a.vt = reinterpret_cast<__half *>(static_cast<char *>(ws) +
-                                           (((size_t)2 * (B + 1) * sizeof(int32_t) + 1023) & ~size_t(1023)));
+  a.tiles = reinterpret_cast<int4 *>(static_cast<char *>(ws) +
+                                     (((size_t)2 * (B + 1) * sizeof(int32_t) + 15) & ~size_t(15)));
+  a.vt = reinterpret_cast<__half *>(static_cast<char *>(ws) + pf_plan_bytes(B, T));
   a.Tp = vt_row(B, T);
   a.B = B;
   a.T = T;

@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 1)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ uint64_t bars[kAttnWarps][kAttnStages];
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int gw = blockIdx.x * kAttnWarps + warp, total_warps = gridDim.x * kAttnWarps;
   uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t *wbuf = base + warp * kAttnStages * kStage;
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 1)
     pi = r - g * n;
   };
 
-  // ---- compute cursor and loader cursor (lane 0 issues the copies) ----
+  // ---- compute cursor and loader cursor (every lane keeps both; one issues the copies) ----
   int cb, cg, cpi;
   locate(start, cb, cg, cpi);
   int cn = pref[cb + 1] - pref[cb], cL = a.seq_lens[cb];
@@ -225,13 +225,15 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 1)
       set_error(a.status, UMIM_ERR_INVALID_ARG);
       c4 = a.n_layers * a.n_pages;
     }
-    uint64_t *bar = &bars[warp][stage];
-    uint8_t *dst = wbuf + stage * kStage;
-    mbar_arrive_expect_tx(bar, kStage);
+    if (elect_one()) {
+      uint64_t *bar = &bars[warp][stage];
+      uint8_t *dst = wbuf + stage * kStage;
+      mbar_arrive_expect_tx(bar, kStage);
 #pragma unroll
-    for (int c = 0; c < NB; ++c) {
-      tma_load_5d(dst + c * 2048, &kv_map, bar, c * 64, 0, lg, 0, c4, pol);
-      tma_load_5d(dst + kTile + c * 2048, &kv_map, bar, c * 64, 0, lg, 1, c4, pol);
+      for (int c = 0; c < NB; ++c) {
+        tma_load_5d(dst + c * 2048, &kv_map, bar, c * 64, 0, lg, 0, c4, pol);
+        tma_load_5d(dst + kTile + c * 2048, &kv_map, bar, c * 64, 0, lg, 1, c4, pol);
+      }
     }
     if (++ld_pos < end && ++lpi == ln) {
       lpi = 0;
@@ -243,9 +245,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 1)
       }
     }
   };
-  if (lane == 0) {
-    for (int s = 0; s < kAttnStages && ld_pos < end; ++s) issue(s);
-  }
+  for (int s = 0; s < kAttnStages && ld_pos < end; ++s) issue(s);
 
   // ---- compute state ----
   const int qr = lane >> 2, qc = lane & 3;      // mma fragment row / column group
@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 1)
     }
     __syncwarp();
     // refill this stage
-    if (lane == 0 && ld_pos < end) issue(stage);
+    if (ld_pos < end) issue(stage);
   }
   flush();
 }

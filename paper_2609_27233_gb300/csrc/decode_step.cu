@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   __shared__ int s_scan[kStepWarps];
   __shared__ int s_last;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int gw = blockIdx.x * kStepWarps + warp;
   const int total_warps = gridDim.x * kStepWarps;
   uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(kStepThreads, 1)
 
   if (start < end) {
     const uint64_t pol = policy_evict_first();
-    // ---- loader cursor (lane 0 issues the copies) ----
+    // ---- loader cursor (every lane keeps it; one issues the copies) ----
     int lb, lg, lpi;
     locate(start, lb, lg, lpi);
     SeqStep lst = seq_step(a, lb);
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(kStepThreads, 1)
       uint64_t *bar = &bars[warp][stage];
       uint8_t *dst = wbuf + stage * kStage;
       if (lst.slot >= 0 && lpi == lst.slot / kPageSize && lst.slot % kPageSize == 0) {
-        mbar_arrive(bar);   // only the new entry in this unit: nothing to copy
+        if (elect_one()) mbar_arrive(bar);   // only the new entry in this unit: nothing to copy
       } else {
         const int page = in_bounds(lpi, a.max_pages, a.status, kSiteStepTable)
                              ? a.block_table[(int64_t)lb * a.max_pages + lpi] : -1;
@@ -272,11 +272,13 @@ __global__ void __launch_bounds__(kStepThreads, 1)
           set_error(a.status, UMIM_ERR_INVALID_ARG);   // a coordinate past the last page reads zeros
           c4 = a.n_layers * a.n_pages;
         }
-        mbar_arrive_expect_tx(bar, kStage);
+        if (elect_one()) {
+          mbar_arrive_expect_tx(bar, kStage);
 #pragma unroll
-        for (int c = 0; c < NB; ++c) {
-          tma_load_5d(dst + c * 2048, &kv_map, bar, c * 64, 0, lg, 0, c4, pol);
-          tma_load_5d(dst + kTile + c * 2048, &kv_map, bar, c * 64, 0, lg, 1, c4, pol);
+          for (int c = 0; c < NB; ++c) {
+            tma_load_5d(dst + c * 2048, &kv_map, bar, c * 64, 0, lg, 0, c4, pol);
+            tma_load_5d(dst + kTile + c * 2048, &kv_map, bar, c * 64, 0, lg, 1, c4, pol);
+          }
         }
       }
       // advance the cursor
@@ -295,9 +297,7 @@ __global__ void __launch_bounds__(kStepThreads, 1)
         }
       }
     };
-    if (lane == 0) {
-      for (int s = 0; s < kStepStages && ld_pos < end; ++s) issue(s);
-    }
+    for (int s = 0; s < kStepStages && ld_pos < end; ++s) issue(s);
 
     // ---- compute state ----
     int cb, cg, cpi;
@@ -569,7 +569,7 @@ __global__ void __launch_bounds__(kStepThreads, 1)
       }
       __syncwarp();
       // refill this stage
-      if (lane == 0 && ld_pos < end) issue(stage);
+      if (ld_pos < end) issue(stage);
 
       // advance: the end of a segment flushes it
       if (++cpi == pref[cb + 1] - pref[cb]) {

@@ -415,43 +415,6 @@ __device__ __forceinline__ float2 warp_sum2(float2 v) {
   return v;
 }
 
-// mbarrier wait that sleeps instead of spinning: try_wait with a suspend-time
-// hint (the thread is woken when the phase completes, or after 1 ms), so a
-// warp waiting for the cluster takes no issue slots from warps still
-// computing; bounded by kWaitLimitNs like every wait of the library
-__device__ __forceinline__ bool mbar_try_wait_sleep(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity), "r"(1000000u)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ bool mbar_wait_sleep(uint64_t *bar, uint32_t parity) {
-  const uint32_t a = smem_u32(bar);
-  if (mbar_test_wait(a, parity)) return true;   // a phase already complete costs no suspension
-  if (mbar_try_wait_sleep(a, parity)) return true;
-  const uint64_t t0 = globaltimer();
-  while (true) {
-    if (mbar_try_wait_sleep(a, parity)) return true;
-    if (globaltimer() - t0 > kWaitLimitNs) return false;
-  }
-}
-
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t *>(&p);
@@ -525,7 +488,7 @@ __global__ void __launch_bounds__(T + 32, 1) ce_kernel(CeArgs a) {
   __shared__ __align__(16) float4 xbuf[2][2][NX];     // [stats | sums][row parity][rank * NW + warp]
   __shared__ uint32_t s_tmem;
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = warp_index();
   const uint32_t rank = cluster_ctarank();
   const int C = (int)cluster_size();
   const int cid = (int)cluster_idx(), ncl = (int)cluster_count();
@@ -583,7 +546,7 @@ __global__ void __launch_bounds__(T + 32, 1) ce_kernel(CeArgs a) {
 
   if (warp == NW) {
     // ---- the copies ----
-    if (lane == 0) {
+    if (elect_one()) {
       const uint64_t pol = policy_evict_first();
       int issued = 0, s = 0;
       uint32_t phase = 0;   // of stage s's full barrier for the copy about to be issued

@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   __shared__ int32_t s_bad;
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int num_kb = g.K / BK;
   const int tiles_n = g.N / BN;
   const int tiles = tiles_n * ((g.M + BM - 1) / BM);
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         for (int kb = 0; kb < num_kb; ++kb, ++it) {
           const int s = it % STAGES;
           const uint32_t ph = (it / STAGES) & 1;
-          if (!mbar_wait(&empty_bar[s], ph ^ 1)) {
+          if (!mbar_wait_sleep(&empty_bar[s], ph ^ 1)) {
             set_error(g.status, UMIM_ERR_TIMEOUT);
             ok = false;
             break;
@@ -159,13 +159,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = g.idesc;
       uint32_t it = 0, local = 0;
       bool ok = true;
       for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++local) {
         const uint32_t buf = local & 1, aph = (local >> 1) & 1;
-        if (!mbar_wait(&acc_empty[buf], aph ^ 1)) {
+        if (!mbar_wait_sleep(&acc_empty[buf], aph ^ 1)) {
           set_error(g.status, UMIM_ERR_TIMEOUT);
           break;
         }
@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         for (int kb = 0; kb < num_kb; ++kb, ++it) {
           const int s = it % STAGES;
           const uint32_t ph = (it / STAGES) & 1;
-          if (!mbar_wait(&full_bar[s], ph)) {
+          if (!mbar_wait_sleep(&full_bar[s], ph)) {
             set_error(g.status, UMIM_ERR_TIMEOUT);
             ok = false;
             break;
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       const int m0 = (tile / tiles_n) * BM, n0 = (tile % tiles_n) * BN;
       const uint32_t buf = local & 1, aph = (local >> 1) & 1;
       const int row = m0 + q * 32 + lane;
-      if (!mbar_wait(&acc_full[buf], aph)) {
+      if (!mbar_wait_sleep(&acc_full[buf], aph)) {
         set_error(g.status, UMIM_ERR_TIMEOUT);
         break;
       }
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kSkThreads, 1)
   __shared__ float2 s_stats[BN / kSkGroup][BM];   // rank 0's: (mean, M2) of every 32 columns of a row
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int split = (int)cluster_size(), rank = (int)cluster_ctarank();
   const int tiles_n = g.N / BN, tile = blockIdx.x / split;
   const int m0 = (tile / tiles_n) * BM, n0 = (tile % tiles_n) * BN;
@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(kSkThreads, 1)
   };
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       const uint64_t pol_a = policy_evict_last(), pol_b = policy_evict_first();
       auto load_b = [&](int i) {
         mbar_arrive_expect_tx(&full_bar[i % STAGES], kStageBytes);
@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(kSkThreads, 1)
       for (int i = 0; i < nkb; ++i) {
         const int s = i % STAGES;
         if (i >= STAGES) {
-          if (!mbar_wait(&empty_bar[s], ((i / STAGES) & 1) ^ 1)) {
+          if (!mbar_wait_sleep(&empty_bar[s], ((i / STAGES) & 1) ^ 1)) {
             set_error(g.status, UMIM_ERR_TIMEOUT);
             break;
           }
@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(kSkThreads, 1)
         ++issued;
       }
       // every copy has landed before the ring is reused or the CTA leaves (bounded)
-      for (int i = max(0, issued - STAGES); i < issued; ++i) mbar_wait(&full_bar[i % STAGES], (i / STAGES) & 1);
+      for (int i = max(0, issued - STAGES); i < issued; ++i) mbar_wait_sleep(&full_bar[i % STAGES], (i / STAGES) & 1);
     }
     __syncwarp();
     if (blockIdx.x == 0) {   // the call's last product: take over what the kernels before found
@@ -430,10 +430,10 @@ __global__ void __launch_bounds__(kSkThreads, 1)
       if (any) *reinterpret_cast<volatile int32_t *>(&s_bad) = 1;
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       for (int i = 0; i < nkb; ++i) {
         const int s = i % STAGES;
-        if (!mbar_wait(CONV ? &conv_bar[s] : &full_bar[s], (i / STAGES) & 1)) {
+        if (!mbar_wait_sleep(CONV ? &conv_bar[s] : &full_bar[s], (i / STAGES) & 1)) {
           set_error(g.status, UMIM_ERR_TIMEOUT);
           break;
         }
@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(kSkThreads, 1)
       uint32_t inf = 0;
       for (int i = 0; i < nkb; ++i) {
         const int s = i % STAGES;
-        if (!__all_sync(0xffffffffu, mbar_wait(&full_bar[s], (i / STAGES) & 1))) {
+        if (!__all_sync(0xffffffffu, mbar_wait_sleep(&full_bar[s], (i / STAGES) & 1))) {
           set_error(g.status, UMIM_ERR_TIMEOUT);
           break;
         }
@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(kSkThreads, 1)
       }
       if (inf & 0x80008000u) flag_range(&s_bad, g.status);
     }
-    if (!__all_sync(0xffffffffu, mbar_wait(&acc_bar, 0))) {
+    if (!__all_sync(0xffffffffu, mbar_wait_sleep(&acc_bar, 0))) {
       set_error(g.status, UMIM_ERR_TIMEOUT);
     } else if (m0 + q * 32 < g.M) {
       tc_fence_after();

@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(kPfThreads, 2)
   __shared__ int s_abort;
   __shared__ int4 s_rec[4];   // the records of the CTA's units k & 3 (written by the copy thread before it loads Q)
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(pf_raw) + 1023) & ~uintptr_t(1023));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     s_abort = 0;
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(kPfThreads, 2)
   };
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       const uint64_t pol_q = policy_evict_first(), pol_kv = policy_evict_last();
       // K runs kPfKStages - 1 tiles ahead of V^T: a K load never waits behind
       // the P V product that frees a V^T stage
@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(kPfThreads, 2)
     }
   } else if (warp == 1) {
     // ---- S = Q K(i)^T into S buffer (tile counter) & 1, once the P V product that read that buffer is done ----
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc_s = idesc_f32acc(kPfRows, kPfKeys, false);
       bool ok = true;
       int nt = 0, k_unit = 0;   // tiles and units so far
@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(kPfThreads, 2)
     // stage and S(i)'s buffer.  A separate issuing thread, so that a P V product never waits behind
     // an S product that waits for the previous P V.  A unit's first product overwrites O once the
     // previous unit's epilogue has read it ----
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc_o = idesc_f32acc(kPfRows, D, true);   // P and V^T in fp16
       bool ok = true;
       int nt = 0, k_unit = 0;

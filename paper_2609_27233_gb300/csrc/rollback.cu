@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
   __shared__ int64_t s_toff[kSmemLanes];
   __shared__ int32_t s_tlh[kSmemLanes];
   __shared__ __align__(8) float s_w[ROPE ? D / 2 : 2];   // RoPE angular frequencies
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, wid = warp_index();
   const int nm = gridDim.x * kBulkMovers;
   uint8_t *ring = bulk_smem + (size_t)wid * kBulkStages * TILE;
 
@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
       m.ra = m.rb = 0;
     }
     uint64_t *bar = &bars[wid][st];
-    if (lane == 0) mbar_arrive_expect_tx(bar, (uint32_t)((m.rb - m.ra) * ROW));
+    if (elect_one()) mbar_arrive_expect_tx(bar, (uint32_t)((m.rb - m.ra) * ROW));
     __syncwarp();
     // slots whose sources are consecutive rows of one old page form a run,
     // copied by the run's first lane in one piece
@@ -414,8 +414,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
     }
     // the reader rows' counts as they are now (counts only grow)
     m.seen = a.n_lanes;
-    if (lane == 0)
-      for (int rw = m.dlo; rw <= m.dhi; ++rw) m.seen = min(m.seen, ld_relaxed(&pd.dep[rw].landed));
+    for (int rw = m.dlo; rw <= m.dhi; ++rw) m.seen = min(m.seen, ld_relaxed(&pd.dep[rw].landed));
   };
   // RoPE: a moved key (shift r > 0) is rotated in shared memory by -r w_m on the
   // pairs (m, m + rotary_dim/2): x' = x cos + y sin, y' = y cos - x sin, with the
@@ -530,7 +529,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
   auto step = [&](int k, Unit &cur, int st, Unit &nxt, int st_nxt) -> bool {
     if (k + S - 1 < my_units) {
       nxt = Nx;
-      if (lane == 0) bulk_wait_read_all();   // unit k - 1's store has read stage st_nxt
+      if (elect_one()) bulk_wait_read_all();   // unit k - 1's store has read stage st_nxt
       __syncwarp();
       issue(nxt, st_nxt);
       ++issued;
@@ -543,7 +542,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
       __syncwarp();
     }
     bool ok = true;
-    if (lane == 0 && cur.valid) {
+    if (cur.valid && elect_one()) {   // (the same lane every time: it waits for its own stores)
       // the unit's rows are in shared memory, so its reads of the old pages are done: count it
       // (relaxed: a release would also wait for this thread's earlier bulk stores to reach memory)
       asm volatile("red.relaxed.gpu.global.add.s32 [%0], 1;" ::"l"(&pd.dep[cur.idx].landed) : "memory");
@@ -554,7 +553,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
                  (uint32_t)((cur.rb - cur.ra) * ROW), pol_store);
       }
     }
-    return __shfl_sync(0xffffffffu, ok, 0);
+    return __all_sync(0xffffffffu, ok) != 0;
   };
   int done = 0;   // units whose rows landed
   bool ok = true;
@@ -575,7 +574,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
     for (int u = done; u < issued; ++u)
       mbar_wait(&bars[wid][u % kBulkStages], (uint32_t)(u / kBulkStages) & 1u);
   }
-  if (lane == 0) bulk_wait_all();
+  if (elect_one()) bulk_wait_all();
   __syncwarp();
   finish_rollback(a, arr, s_last);
 }

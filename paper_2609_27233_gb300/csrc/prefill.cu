@@ -53,7 +53,8 @@ constexpr int kPfKStages = 2;            // K ring (K runs kPfKStages - 1 tiles 
 constexpr int kPfVStages = 2;            // V^T ring
 constexpr int kPfThreads = 224;          // warp 0 TMA, warp 1 S products + tensor memory, warps 2-5 softmax
                                          // (thread = query row), warp 6 P V products
-constexpr int kPfPlanThreads = 1024;
+constexpr int kPfPlanThreads = 1024, kPfVtThreads = 256;
+constexpr int kPfSmemBatch = 2048;       // sequences whose prefix sums a V^T CTA keeps in shared memory
 constexpr uint32_t kPfTmemCols = 256;    // S buffers at 0 and 64, O at 128: two CTAs per SM
 
 struct PfArgs {
@@ -70,22 +71,21 @@ struct PfArgs {
   int32_t *status;
 };
 
-// One block: validates cu_seqlens, writes the prefix sums of query tiles and
-// of sequence lengths rounded up to 64 keys.
-__global__ void __launch_bounds__(kPfPlanThreads) prefill_plan_kernel(PfArgs a) {
-  griddep_wait();
-  __shared__ int s_wsum[2][kPfPlanThreads / 32];
-  __shared__ int s_err;
+// Exclusive prefix sums over the sequences of query tiles (cu_tiles) and of
+// lengths rounded up to 64 keys (pcu), [0 .. B], by a block of T threads, which
+// also validates cu_seqlens: invalid offsets leave totals of 0, no work at all.
+template <int T>
+__device__ void pf_prefix(const PfArgs &a, int32_t *cu_tiles, int32_t *pcu, bool report) {
+  __shared__ int s_wsum[2][32];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  if (tid == 0) s_err = (a.cu[0] != 0 || a.cu[a.B] > a.T) ? 1 : 0;
-  __syncthreads();
+  int err = a.cu[0] != 0 || a.cu[a.B] > a.T;
   int carry_t = 0, carry_p = 0;
-  for (int base = 0; base < a.B; base += kPfPlanThreads) {
+  for (int base = 0; base < a.B; base += T) {
     const int b = base + tid;
     int n = 0, pk = 0;
     if (b < a.B) {
       const int len = a.cu[b + 1] - a.cu[b];
-      if (len < 0) s_err = 1;
+      if (len < 0) err = 1;
       n = len > 0 ? (len + kPfRows - 1) / kPfRows : 0;
       pk = len > 0 ? (len + kPfKeys - 1) / kPfKeys * kPfKeys : 0;
     }
@@ -104,7 +104,8 @@ __global__ void __launch_bounds__(kPfPlanThreads) prefill_plan_kernel(PfArgs a) 
     }
     __syncthreads();
     int bt = 0, tt = 0, bp = 0, tp = 0;
-    for (int w = 0; w < kPfPlanThreads / 32; ++w) {
+#pragma unroll
+    for (int w = 0; w < T / 32; ++w) {
       if (w < wid) {
         bt += s_wsum[0][w];
         bp += s_wsum[1][w];
@@ -113,18 +114,26 @@ __global__ void __launch_bounds__(kPfPlanThreads) prefill_plan_kernel(PfArgs a) 
       tp += s_wsum[1][w];
     }
     if (b < a.B) {
-      a.cu_tiles[b] = carry_t + bt + it - n;
-      a.pcu[b] = carry_p + bp + ip - pk;
+      cu_tiles[b] = carry_t + bt + it - n;
+      pcu[b] = carry_p + bp + ip - pk;
     }
     carry_t += tt;
     carry_p += tp;
     __syncthreads();
   }
+  err = __syncthreads_or(err);
   if (tid == 0) {
-    if (s_err) set_error(a.status, UMIM_ERR_INVALID_ARG);
-    a.cu_tiles[a.B] = s_err ? 0 : carry_t;   // invalid offsets: no work at all
-    a.pcu[a.B] = s_err ? 0 : carry_p;
+    if (err && report) set_error(a.status, UMIM_ERR_INVALID_ARG);
+    cu_tiles[a.B] = err ? 0 : carry_t;
+    pcu[a.B] = err ? 0 : carry_p;
   }
+  __syncthreads();
+}
+
+// more than kPfSmemBatch sequences: the prefix sums in a kernel of its own (one block)
+__global__ void __launch_bounds__(kPfPlanThreads) prefill_plan_kernel(PfArgs a) {
+  griddep_wait();
+  pf_prefix<kPfPlanThreads>(a, a.cu_tiles, a.pcu, true);
 }
 
 // last index b in [0, B) with key[b] <= x
@@ -139,47 +148,75 @@ __device__ __forceinline__ int pf_find(const int32_t *key, int B, int x) {
 }
 
 // V^T: vt[g][d][pcu[b] + t] = v[cu[b] + t][g][d] for t < len_b, 0 up to the
-// next multiple of 64.  One CTA per 64 padded keys and KV head, through a
-// shared-memory tile.  The CTAs of KV head 0 whose keys start a query tile also
-// write that tile's record.
-template <int D>
-__global__ void __launch_bounds__(256) vt_kernel(PfArgs a) {
+// next multiple of 64.  CTAs walk the (64 padded keys, KV head) blocks, each
+// through a shared-memory tile.  The blocks of KV head 0 whose keys start a
+// query tile also write that tile's record.  With PLAN the CTAs derive the
+// prefix sums themselves, in shared memory, once each: as a kernel before this
+// one they cost a launch and a trip through memory (five short prompts: 12.7 ->
+// 10.0 us; 64 of 1500 rows: both kernels 80 -> 71 us).
+template <int D, bool PLAN>
+__global__ void __launch_bounds__(kPfVtThreads) vt_kernel(PfArgs a) {
   griddep_wait();
   __shared__ uint32_t tile[kPfKeys][D / 2 + 1];   // bf16 pairs, padded against bank conflicts
-  const int k0 = blockIdx.x * kPfKeys, g = blockIdx.y;
-  if (k0 >= a.pcu[a.B]) return;
-  const int b = pf_find(a.pcu, a.B, k0);
-  const int len = a.cu[b + 1] - a.cu[b];
-  const int t0 = k0 - a.pcu[b];
-  if (g == 0 && threadIdx.x == 0 && t0 % kPfRows == 0)
-    a.tiles[a.cu_tiles[b] + t0 / kPfRows] = make_int4(a.cu[b], len, t0, a.pcu[b]);
-  constexpr int CPR = D / 8;   // 16-byte chunks per key row
-  for (int i = threadIdx.x; i < kPfKeys * CPR; i += blockDim.x) {
-    const int r = i / CPR, c = i % CPR;
-    uint4 u = make_uint4(0, 0, 0, 0);
-    if (t0 + r < len)
-      u = __ldg(reinterpret_cast<const uint4 *>(a.v + ((int64_t)(a.cu[b] + t0 + r) * a.Hkv + g) * D) + c);
-    tile[r][4 * c] = u.x;
-    tile[r][4 * c + 1] = u.y;
-    tile[r][4 * c + 2] = u.z;
-    tile[r][4 * c + 3] = u.w;
+  extern __shared__ int32_t s_plan[];             // PLAN: the prefix sums, [B + 1] each
+  const int32_t *cu_tiles = a.cu_tiles, *pcu = a.pcu;
+  if (PLAN) {
+    pf_prefix<kPfVtThreads>(a, s_plan, s_plan + a.B + 1, blockIdx.x == 0);
+    cu_tiles = s_plan;
+    pcu = s_plan + a.B + 1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.cu_tiles[a.B] = cu_tiles[a.B];   // for the attention kernel
   }
-  __syncthreads();
-  // each thread writes 8 keys of one d row (16 bytes), converted to fp16
-  bool too_big = false;
-  for (int i = threadIdx.x; i < D * (kPfKeys / 8); i += blockDim.x) {
-    const int d = i / (kPfKeys / 8), c = i % (kPfKeys / 8);
-    uint32_t w[4];
+  const int blocks = pcu[a.B] / kPfKeys * a.Hkv;
+  constexpr int CPR = D / 8;                             // 16-byte chunks per key row
+  constexpr int NU = kPfKeys * CPR / kPfVtThreads;       // chunks a thread loads
+  uint4 u[NU];
+  // a block's rows; the next block's are loaded while this one is written
+  auto load = [&](int it) {
+    const int k0 = it / a.Hkv * kPfKeys, g = it % a.Hkv;
+    const int b = pf_find(pcu, a.B, k0);
+    const int first = a.cu[b], len = a.cu[b + 1] - first;
+    const int t0 = k0 - pcu[b];
+    if (g == 0 && threadIdx.x == 0 && t0 % kPfRows == 0)
+      a.tiles[cu_tiles[b] + t0 / kPfRows] = make_int4(first, len, t0, pcu[b]);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t x0 = tile[8 * c + 2 * j][d >> 1], x1 = tile[8 * c + 2 * j + 1][d >> 1];
-      const float f0 = __uint_as_float((d & 1) ? (x0 & 0xffff0000u) : (x0 << 16));
-      const float f1 = __uint_as_float((d & 1) ? (x1 & 0xffff0000u) : (x1 << 16));
-      too_big |= !(fabsf(f0) < 65504.f) || !(fabsf(f1) < 65504.f);
-      const __half2 hh = __floats2half2_rn(f0, f1);
-      w[j] = *reinterpret_cast<const uint32_t *>(&hh);
+    for (int k = 0; k < NU; ++k) {
+      const int i = threadIdx.x + k * kPfVtThreads, r = i / CPR, c = i % CPR;
+      u[k] = make_uint4(0, 0, 0, 0);
+      if (t0 + r < len)
+        u[k] = __ldg(reinterpret_cast<const uint4 *>(a.v + ((int64_t)(first + t0 + r) * a.Hkv + g) * D) + c);
     }
-    *reinterpret_cast<uint4 *>(a.vt + ((int64_t)g * D + d) * a.Tp + k0 + 8 * c) = make_uint4(w[0], w[1], w[2], w[3]);
+  };
+  bool too_big = false;
+  if ((int)blockIdx.x < blocks) load(blockIdx.x);
+  for (int it = blockIdx.x; it < blocks; it += gridDim.x) {
+    const int k0 = it / a.Hkv * kPfKeys, g = it % a.Hkv;
+#pragma unroll
+    for (int k = 0; k < NU; ++k) {
+      const int i = threadIdx.x + k * kPfVtThreads, r = i / CPR, c = i % CPR;
+      tile[r][4 * c] = u[k].x;
+      tile[r][4 * c + 1] = u[k].y;
+      tile[r][4 * c + 2] = u[k].z;
+      tile[r][4 * c + 3] = u[k].w;
+    }
+    __syncthreads();
+    if (it + (int)gridDim.x < blocks) load(it + gridDim.x);
+    // each thread writes 8 keys of one d row (16 bytes), converted to fp16
+    for (int i = threadIdx.x; i < D * (kPfKeys / 8); i += kPfVtThreads) {
+      const int d = i / (kPfKeys / 8), c = i % (kPfKeys / 8);
+      uint32_t w[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t x0 = tile[8 * c + 2 * j][d >> 1], x1 = tile[8 * c + 2 * j + 1][d >> 1];
+        const float f0 = __uint_as_float((d & 1) ? (x0 & 0xffff0000u) : (x0 << 16));
+        const float f1 = __uint_as_float((d & 1) ? (x1 & 0xffff0000u) : (x1 << 16));
+        too_big |= !(fabsf(f0) < 65504.f) || !(fabsf(f1) < 65504.f);
+        const __half2 hh = __floats2half2_rn(f0, f1);
+        w[j] = *reinterpret_cast<const uint32_t *>(&hh);
+      }
+      *reinterpret_cast<uint4 *>(a.vt + ((int64_t)g * D + d) * a.Tp + k0 + 8 * c) =
+          make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    __syncthreads();   // the tile is filled again
   }
   if (too_big) set_error(a.status, UMIM_ERR_UNSUPPORTED);   // |v| outside fp16's range (or not finite)
 }
@@ -689,12 +726,20 @@ umim_status prefill_attention(const void *q, const void *k, const void *v, int T
       !encode_3d(enc, &km, k, D, Hkv, T, (uint64_t)D * 2, (uint64_t)Hkv * D * 2, 64, 1, kPfKeys) ||
       !encode_3d(enc, &vm, a.vt, a.Tp, D, Hkv, (uint64_t)a.Tp * 2, (uint64_t)D * a.Tp * 2, kPfKeys, D, 1, true))
     return UMIM_ERR_CUDA;
-  trace_mark(stream, "prefill.plan");
-  if (launch_pdl(prefill_plan_kernel, dim3(1), dim3(kPfPlanThreads), 0, stream, a) != cudaSuccess)
-    return UMIM_ERR_CUDA;
+  const bool plan = B <= kPfSmemBatch;
+  if (!plan) {
+    trace_mark(stream, "prefill.plan");
+    if (launch_pdl(prefill_plan_kernel, dim3(1), dim3(kPfPlanThreads), 0, stream, a) != cudaSuccess)
+      return UMIM_ERR_CUDA;
+  }
   trace_mark(stream, "prefill.v_transpose");
-  auto vk = D == 128 ? vt_kernel<128> : vt_kernel<64>;
-  if (launch_pdl(vk, dim3((unsigned)(a.Tp / kPfKeys), (unsigned)Hkv), dim3(256), 0, stream, a) != cudaSuccess)
+  auto vk = plan ? (D == 128 ? vt_kernel<128, true> : vt_kernel<64, true>)
+                 : (D == 128 ? vt_kernel<128, false> : vt_kernel<64, false>);
+  const int64_t vt_blocks = a.Tp / kPfKeys * Hkv;
+  // eight CTAs an SM are resident (six took 82 us for 96 000 rows of 8 heads, eight 71)
+  const unsigned vt_grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(vt_blocks, 8LL * std::max(num_sms, 1)));
+  if (launch_pdl(vk, dim3(vt_grid), dim3(kPfVtThreads), plan ? 2 * sizeof(int32_t) * ((size_t)B + 1) : 0, stream, a) !=
+      cudaSuccess)
     return UMIM_ERR_CUDA;
   auto kern = D == 128 ? prefill_tc_kernel<128> : prefill_tc_kernel<64>;
   const size_t smem = (size_t)(D == 128 ? PfSmem<128>::kTotal : PfSmem<64>::kTotal) + 1024;

@@ -1,0 +1,29 @@
+"""Prefill attention's plan at its edges (prefix sums in every V^T CTA up to 2048 sequences, 256 a pass; a kernel of its
+own beyond), and lengths that end on and next to the 64-key and 128-row tiles, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads as W
+from helpers import dev, float_close, umim
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,hi", [(1, 129), (255, 5), (256, 5), (257, 5), (2048, 3), (2049, 3), (12, 260)])
+def test_many_prompts_match_oracle(B, hi):
+    m, dv = umim(), dev()
+    r = np.random.default_rng(B)
+    lens = r.integers(0, hi + 1, size=B)
+    lens[:5] = ([hi, 127, 128, 129, 64] if hi > 128 else [hi] * 5)[:B]
+    lens[-1] = hi
+    T = int(lens.sum())
+    q, k, v = (W.bf16_normal((T, h, 64), 1.0, 300 + B + h, dv) for h in (2, 1, 1))
+    cu = torch.tensor(np.concatenate([[0], np.cumsum(lens)]), dtype=torch.int32, device=dv)
+    status = m.new_status(dv)
+    out = m.umim_prefill_attention(q, k, v, cu, dev_status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    want = oracle.prefill_attention(W.bits(q), W.bits(k), W.bits(v), cu.cpu().numpy())
+    float_close(out.cpu().double().numpy(), want)

@@ -1,210 +1,14 @@
-// Span metadata kernel: one block per sequence validates its spans and scans
-// (k_i - 1); the last block to finish builds the prefix sums over sequences.
-#include "plan.cuh"
+// The span metadata kernel of prompt compaction, and of rollbacks whose map is a
+// kernel of its own.
+#include "plan_block.cuh"
 
 namespace umim {
 namespace {
 
-constexpr int kPlanThreads = 1024;
-
-// Spans a thread takes per pass, consecutive ones: their loads are in flight
-// together and a sequence of up to 8192 spans needs one block-wide scan.  With
-// one span a thread, four sequences of 4369 spans took five passes of loads,
-// scan and barriers (18.4 us, now 16.2 us).
-constexpr int kPlanItems = 8;
-
-// Inclusive block-wide scan of four sums at once; every thread gets the totals.
-__device__ int4 block_scan_incl(int4 v, int4 &total) {
-  __shared__ int4 warp_sums[kPlanThreads / 32];
-  static_assert(kPlanThreads / 32 == 32, "one lane per warp");
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  auto warp_scan = [&](int4 x) {
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int4 y = make_int4(__shfl_up_sync(0xffffffffu, x.x, o), __shfl_up_sync(0xffffffffu, x.y, o),
-                               __shfl_up_sync(0xffffffffu, x.z, o), __shfl_up_sync(0xffffffffu, x.w, o));
-      if (lane >= o) {
-        x.x += y.x;
-        x.y += y.y;
-        x.z += y.z;
-        x.w += y.w;
-      }
-    }
-    return x;
-  };
-  v = warp_scan(v);
-  if (lane == 31) warp_sums[w] = v;
-  __syncthreads();
-  const int4 s = warp_scan(warp_sums[lane]);   // every warp scans the warps' sums
-  auto from = [&](int src) {
-    return make_int4(__shfl_sync(0xffffffffu, s.x, src), __shfl_sync(0xffffffffu, s.y, src),
-                     __shfl_sync(0xffffffffu, s.z, src), __shfl_sync(0xffffffffu, s.w, src));
-  };
-  total = from(31);
-  const int4 add = from(w > 0 ? w - 1 : 0);
-  if (w > 0) {
-    v.x += add.x;
-    v.y += add.y;
-    v.z += add.z;
-    v.w += add.w;
-  }
-  __syncthreads();
-  return v;
-}
-
-// The same for one sum.
-__device__ int block_scan_incl(int v, int &total) {
-  __shared__ int warp_sums[kPlanThreads / 32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  auto warp_scan = [&](int x) {
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    return x;
-  };
-  v = warp_scan(v);
-  if (lane == 31) warp_sums[w] = v;
-  __syncthreads();
-  const int s = warp_scan(warp_sums[lane]);
-  total = __shfl_sync(0xffffffffu, s, 31);
-  const int add = __shfl_sync(0xffffffffu, s, w > 0 ? w - 1 : 0);
-  __syncthreads();
-  return v + (w > 0 ? add : 0);
-}
-
 __global__ void __launch_bounds__(kPlanThreads) span_plan_kernel(PlanArgs a, PlanArrays arr) {
   griddep_wait();
-  const int b = blockIdx.x;
-  __shared__ int s_err, s_last;
-  if (threadIdx.x == 0) {
-    s_err = 0;
-    s_last = 0;
-  }
-  __syncthreads();
-  const int L = a.seq_lens ? a.seq_lens[b] : a.fixed_len;
-  const int lo = a.span_offsets[b], hi = a.span_offsets[b + 1];
-  bool bad = (lo < 0) || (hi < lo) || (hi > a.S) || (L < 0);
-  if (a.block_table && (int64_t)L > (int64_t)a.max_pages * kPageSize) bad = true;
-  if (bad && threadIdx.x == 0) s_err = 1;
-  int removed = 0;   // by the spans of the passes so far
-  if (!bad) {        // (the same in every thread)
-    if (a.block_table) {
-      const int np = ceil_div(L, kPageSize);
-      for (int p = threadIdx.x; p < np; p += kPlanThreads) {
-        const int pg = a.block_table[(int64_t)b * a.max_pages + p];
-        if (pg < 0 || pg >= a.n_pages) s_err = 1;
-      }
-    }
-    for (int base = lo; base < hi; base += kPlanThreads * kPlanItems) {
-      const int per = min(kPlanItems, ceil_div(hi - base, kPlanThreads));
-      const int i0 = min(base + (int)threadIdx.x * per, hi), n = min(per, hi - i0);
-      int s[kPlanItems], k[kPlanItems];
-#pragma unroll
-      for (int u = 0; u < kPlanItems; ++u)
-        if (u < n) {
-          s[u] = a.span_start[i0 + u];
-          k[u] = a.span_len[i0 + u];
-        }
-      // the end of the span before: positions up to it are taken
-      int64_t end = n > 0 && i0 > lo ? (int64_t)a.span_start[i0 - 1] + a.span_len[i0 - 1] : 0;
-      int sum = 0;
-      bool ok = true;
-#pragma unroll
-      for (int u = 0; u < kPlanItems; ++u)
-        if (u < n) {
-          const bool good = k[u] >= 1 && s[u] >= 0 && (int64_t)s[u] + k[u] <= L && end <= s[u] &&
-                            !(a.max_span_len > 0 && k[u] > a.max_span_len);
-          end = (int64_t)s[u] + k[u];
-          ok = ok && good;
-          sum += good ? k[u] - 1 : 0;
-        }
-      if (!ok) s_err = 1;
-      int tot;
-      int r = removed + block_scan_incl(sum, tot) - sum;   // removed before this thread's spans
-#pragma unroll
-      for (int u = 0; u < kPlanItems; ++u)
-        if (u < n) {
-          arr.new_idx[i0 + u] = s[u] - r;
-          r += k[u] - 1;
-          arr.r_incl[i0 + u] = r;
-        }
-      removed += tot;
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const int err = s_err;
-    const int Lp = err ? L : L - removed;
-    arr.seq_L[b] = L;
-    arr.seq_Lp[b] = Lp;
-    int fp = 0, nd = 0;
-    if (!err && hi > lo) {
-      fp = a.span_start[lo] / kPageSize;
-      nd = ceil_div(Lp, kPageSize) - fp;
-    }
-    arr.first_page[b] = fp;
-    arr.n_dest[b] = nd;
-    if (err) atomicOr(&arr.hdr->error, 1);
-    __threadfence();
-    const int done = atomicAdd(&arr.hdr->blocks_done, 1);
-    s_last = (done == (int)gridDim.x - 1);
-  }
-  __syncthreads();
-  if (!s_last) return;
-
-  // ---- last block: prefix sums over sequences, per-call header reset ----
-  __threadfence();
-  const int err = atomicOr(&arr.hdr->error, 0);
-  int cu_units = 0, cu_rows = 0, cu_freed = 0, cu_active = 0;
-  __shared__ int s_max_dest;
-  if (threadIdx.x == 0) s_max_dest = 0;
-  __syncthreads();
-  for (int j = threadIdx.x; j < a.B; j += kPlanThreads) atomicMax(&s_max_dest, arr.n_dest[j]);
-  for (int base = 0; base < a.B; base += kPlanThreads) {
-    const int j = base + threadIdx.x;
-    int u = 0, r = 0, f = 0;
-    if (j < a.B) {
-      const int L = arr.seq_L[j], Lp = arr.seq_Lp[j];
-      u = a.n_lanes * arr.n_dest[j];
-      r = Lp;
-      f = ceil_div(L, kPageSize) - ceil_div(Lp, kPageSize);
-    }
-    const int act = (j < a.B && arr.n_dest[j] > 0) ? 1 : 0;
-    int4 tot;
-    const int4 incl = block_scan_incl(make_int4(u, r, f, act), tot);
-    if (j < a.B) {
-      arr.unit_base[j] = cu_units + incl.x - u;
-      arr.row_base[j] = cu_rows + incl.y - r;
-      arr.freed_base[j] = cu_freed + incl.z - f;
-      if (act) arr.active[cu_active + incl.w - 1] = j;
-      if (a.cu_seqlens_out && !err) a.cu_seqlens_out[j] = cu_rows + incl.y - r;
-    }
-    cu_units += tot.x;
-    cu_rows += tot.y;
-    cu_freed += tot.z;
-    cu_active += tot.w;
-  }
-  if (threadIdx.x == 0) {
-    arr.unit_base[a.B] = cu_units;
-    arr.row_base[a.B] = cu_rows;
-    arr.freed_base[a.B] = cu_freed;
-    if (a.cu_seqlens_out && !err) a.cu_seqlens_out[a.B] = cu_rows;
-    PlanHeader *h = arr.hdr;
-    h->total_units = err ? 0 : cu_units;
-    h->total_rows = cu_rows;
-    h->max_dest = err ? 0 : s_max_dest;
-    h->n_active = err ? 0 : cu_active;
-    h->skip = err ? 1 : 0;
-    h->epoch = h->epoch + 1;
-    h->ticket = 0;
-    h->done_ctas = 0;
-    h->blocks_done = 0;
-    h->error = 0;
-    if (err) set_error(a.status, UMIM_ERR_INVALID_ARG);
-    __threadfence();
-  }
+  const PlanSeq q = plan_sequence(a, arr, nullptr);
+  if (q.last) plan_totals(a, arr);
 }
 
 }  // namespace

@@ -22,7 +22,7 @@
 // One pass: each moved byte is read once and written once.
 #include <algorithm>
 
-#include "plan.cuh"
+#include "plan_block.cuh"
 
 namespace umim {
 namespace {
@@ -75,6 +75,67 @@ struct PageDesc {
   RowDep *dep;     // [rows]
   int32_t *shift;  // [rows][16] r of a moved kept entry (positions removed before it), else 0
 };
+
+// The spans that may be the last at or before a position: by compressed index
+// (for the entries of compacted pages) and by start (for old entries).
+struct SpanWindow {
+  const int32_t *new_idx, *new_r;   // [n_new] ascending
+  int n_new, first_new;             // the number of the first span among all
+  const int32_t *start, *end, *r;   // [n_start]
+  int n_start;
+};
+
+// One thread per slot of compacted page k of sequence b (16 threads together):
+// where its entry comes from, and which compacted rows read the old entries of
+// the page.  Row k of sequence b is row b * max_pages + k of the descriptions.
+__device__ __forceinline__ void map_slot(const MoveArgs &a, const PageDesc &pd, int D, const SpanWindow &w, int b,
+                                         int fp, int k, int slot, int nd, int L, int Lp, int first) {
+  const int idx = b * a.max_pages + k;
+  int64_t src = kNoWrite;
+  int32_t shift = 0;
+  int rd_lo = INT32_MAX, rd_hi = -1;
+  if (k < nd) {
+    const int32_t *bt = a.block_table + (int64_t)b * a.max_pages;
+    const int64_t page_stride = (int64_t)kPageSize * D * a.n_kv_heads * 2;
+    const int j = (fp + k) * kPageSize + slot;
+    if (j < Lp && j >= first) {
+      const int i = upper_index(w.new_idx, 0, w.n_new, j);
+      if (i >= 0) {
+        if (w.new_idx[i] == j) {
+          src = -(int64_t)(w.first_new + i) - 1;
+        } else {
+          const int t = j + w.new_r[i];
+          if (t != j && in_bounds(t / kPageSize, a.max_pages, a.status, kSiteRollbackMapTable)) {
+            src = (int64_t)bt[t / kPageSize] * page_stride + (t % kPageSize) * D;
+            shift = t - j;
+          }
+        }
+      }
+    }
+    // the old entry t in this slot of the page: the compacted row that reads it
+    const int t = j;
+    if (t < L) {
+      const int i = upper_index(w.start, 0, w.n_start, t);
+      if (i >= 0 && t >= w.end[i] && w.r[i] > 0) rd_lo = rd_hi = (t - w.r[i]) / kPageSize - fp;
+    }
+  }
+  for (int o = 8; o > 0; o >>= 1) {   // over the row's 16 slots
+    rd_lo = min(rd_lo, __shfl_xor_sync(0xffffffffu, rd_lo, o, 16));
+    rd_hi = max(rd_hi, __shfl_xor_sync(0xffffffffu, rd_hi, o, 16));
+  }
+  if (k >= nd) return;
+  pd.src[(int64_t)idx * kPageSize + slot] = src;
+  if (a.rope_inv_freq) pd.shift[(int64_t)idx * kPageSize + slot] = shift;
+  if (slot == 0) {
+    rd_hi = min(rd_hi, k - 1);   // the row itself reads only its own units' columns
+    RowDep d;
+    d.lo = rd_lo <= rd_hi ? idx - k + rd_lo : 1;
+    d.hi = rd_lo <= rd_hi ? idx - k + rd_hi : 0;
+    d.landed = 0;
+    d.pad = 0;
+    pd.dep[idx] = d;
+  }
+}
 
 // Sixteen threads per (sequence, compacted page), sixteen pages per CTA: where
 // each of a page's 16 entries comes from (kNoWrite: the entry does not move),
@@ -134,54 +195,33 @@ __global__ void __launch_bounds__(kMapThreads) rollback_map_kernel(MoveArgs a, P
   }
   const int k = k0 + (threadIdx.x >> 4);
   const int slot = threadIdx.x & 15;
-  const bool row_ok = k < nd;
-  const int idx = arr.unit_base[b] / a.n_lanes + k;
   const int Lp = arr.seq_Lp[b], L = arr.seq_L[b], first = a.span_start[lo];
   __syncthreads();
-  int64_t src = kNoWrite;
-  int32_t shift = 0;
-  int rd_lo = INT32_MAX, rd_hi = -1;
-  if (row_ok) {
-    const int32_t *bt = a.block_table + (int64_t)b * a.max_pages;
-    const int64_t page_stride = (int64_t)kPageSize * D * a.n_kv_heads * 2;
-    const int j = e0 + (int)threadIdx.x;
-    if (j < Lp && j >= first) {
-      const int i = upper_index(s_new, 0, nw0, j);
-      if (i >= 0) {
-        if (s_new[i] == j) {
-          src = -(int64_t)(w0 + i) - 1;
-        } else {
-          const int t = j + s_newr[i];
-          if (t != j && in_bounds(t / kPageSize, a.max_pages, a.status, kSiteRollbackMapTable)) {
-            src = (int64_t)bt[t / kPageSize] * page_stride + (t % kPageSize) * D;
-            shift = t - j;
-          }
-        }
-      }
-    }
-    // the old entry t in this slot of page p: the compacted row that reads it
-    const int t = j;
-    if (t < L) {
-      const int i = upper_index(s_st, 0, nw1, t);
-      if (i >= 0 && t >= s_end[i] && s_str[i] > 0) rd_lo = rd_hi = (t - s_str[i]) / kPageSize - fp;
-    }
-  }
-  for (int o = 8; o > 0; o >>= 1) {   // over the row's 16 slots
-    rd_lo = min(rd_lo, __shfl_xor_sync(0xffffffffu, rd_lo, o, 16));
-    rd_hi = max(rd_hi, __shfl_xor_sync(0xffffffffu, rd_hi, o, 16));
-  }
-  if (!row_ok) return;
-  pd.src[(int64_t)idx * kPageSize + slot] = src;
-  if (a.rope_inv_freq) pd.shift[(int64_t)idx * kPageSize + slot] = shift;
-  if (slot == 0) {
-    rd_hi = min(rd_hi, k - 1);   // the row itself reads only its own units' columns
-    RowDep d;
-    d.lo = rd_lo <= rd_hi ? idx - k + rd_lo : 1;
-    d.hi = rd_lo <= rd_hi ? idx - k + rd_hi : 0;
-    d.landed = 0;
-    d.pad = 0;
-    pd.dep[idx] = d;
-  }
+  const SpanWindow w{s_new, s_newr, nw0, w0, s_st, s_end, s_str, nw1};
+  map_slot(a, pd, D, w, b, fp, k, slot, nd, L, Lp, first);
+}
+
+// The plan and the map in one kernel, a block per sequence, when the block
+// table has at most kPlanMapPages columns: the spans stay in shared memory and
+// the block maps its pages, 64 a pass.  A kernel of its own for the map costs a
+// launch and the trips above, and pays once a sequence has many passes.
+// MEASURED_PLANMAP
+constexpr int kPlanMapPages = 256;
+constexpr int kPlanMapSpans = kPlanMapPages * kPageSize;   // a span replaces an entry at least
+
+__global__ void __launch_bounds__(kPlanThreads)
+    rollback_plan_map_kernel(PlanArgs pa, MoveArgs a, PlanArrays arr, PageDesc pd, int D) {
+  griddep_wait();
+  extern __shared__ int32_t s_spans[];
+  const SpanCopy c{s_spans, s_spans + kPlanMapSpans, s_spans + 2 * kPlanMapSpans, s_spans + 3 * kPlanMapSpans,
+                   kPlanMapSpans};
+  const PlanSeq q = plan_sequence(pa, arr, &c);
+  const int ns = q.hi - q.lo;
+  const SpanWindow w{c.new_idx, c.r_incl, ns, q.lo, c.start, c.end, c.r_incl, ns};
+  for (int k0 = 0; k0 < q.n_dest; k0 += kPlanThreads / kPageSize)
+    map_slot(a, pd, D, w, blockIdx.x, q.first_page, k0 + (int)threadIdx.x / kPageSize, threadIdx.x % kPageSize,
+             q.n_dest, q.L, q.Lp, c.start[0]);
+  if (q.last) plan_totals(pa, arr);
 }
 
 // The last CTA of the move kernel to finish truncates the block tables,
@@ -305,7 +345,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
   const int row_size = max(1, n_active * a.n_lanes);
   const int max_dest = total > 0 ? hdr->max_dest : 0;
   const int n_slots = max_dest * row_size;
-  const int n_rows = total / a.n_lanes;   // compacted rows of all sequences (debug checks)
+  const int n_rows = a.B * a.max_pages;   // described rows (debug checks)
 
   const bool seq_in_smem = n_active <= kSmemSeqs;
   if (seq_in_smem) {
@@ -313,7 +353,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
       const int b = arr.active[q];
       s_sq[q] = b;
       s_nd[q] = arr.n_dest[b];
-      s_ub[q] = arr.unit_base[b] / a.n_lanes;
+      s_ub[q] = b * a.max_pages;
       s_fp[q] = arr.first_page[b];
     }
   }
@@ -328,7 +368,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
   __syncthreads();
   auto seq_of = [&](int q) { return seq_in_smem ? s_sq[q] : arr.active[q]; };
   auto nd_of = [&](int q) { return seq_in_smem ? s_nd[q] : arr.n_dest[arr.active[q]]; };
-  auto row0_of = [&](int q) { return seq_in_smem ? s_ub[q] : arr.unit_base[arr.active[q]] / a.n_lanes; };
+  auto row0_of = [&](int q) { return seq_in_smem ? s_ub[q] : arr.active[q] * a.max_pages; };
   auto fp_of = [&](int q) { return seq_in_smem ? s_fp[q] : arr.first_page[arr.active[q]]; };
 
   // a unit: where its rows come from and go, and which rows read its page.
@@ -620,9 +660,6 @@ umim_status kv_rollback(const umim_paged_kv *kv, int32_t *block_table, int32_t m
   pa.n_lanes = lanes;
   pa.status = status;
   pa.cu_seqlens_out = nullptr;
-  trace_mark(stream, "rollback.plan");
-  if (launch_span_plan(pa, arr, stream) != cudaSuccess) return UMIM_ERR_CUDA;
-
   MoveArgs ma{};
   ma.pool = static_cast<uint16_t *>(kv->base);
   ma.n_lanes = lanes;
@@ -656,10 +693,23 @@ umim_status kv_rollback(const umim_paged_kv *kv, int32_t *block_table, int32_t m
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1)
     per_sm = 1;
   const int grid = std::max(1, num_sms) * per_sm;   // every CTA resident (cooperative launch)
-  trace_mark(stream, "rollback.map");
-  if (launch_pdl(rollback_map_kernel, dim3((unsigned)std::max(1, ceil_div(max_pages, kMapPages)), (unsigned)B), dim3(kMapThreads), 0,
-                 stream, ma, arr, pd, (int)D) != cudaSuccess)
-    return UMIM_ERR_CUDA;
+  if (max_pages <= kPlanMapPages) {
+    const int plan_smem = 4 * kPlanMapSpans * (int)sizeof(int32_t);
+    if (cudaFuncSetAttribute(rollback_plan_map_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, plan_smem) !=
+        cudaSuccess)
+      return UMIM_ERR_CUDA;
+    trace_mark(stream, "rollback.plan_map");
+    if (launch_pdl(rollback_plan_map_kernel, dim3((unsigned)B), dim3(kPlanThreads), (size_t)plan_smem, stream, pa, ma,
+                   arr, pd, (int)D) != cudaSuccess)
+      return UMIM_ERR_CUDA;
+  } else {
+    trace_mark(stream, "rollback.plan");
+    if (launch_span_plan(pa, arr, stream) != cudaSuccess) return UMIM_ERR_CUDA;
+    trace_mark(stream, "rollback.map");
+    if (launch_pdl(rollback_map_kernel, dim3((unsigned)ceil_div(max_pages, kMapPages), (unsigned)B), dim3(kMapThreads),
+                   0, stream, ma, arr, pd, (int)D) != cudaSuccess)
+      return UMIM_ERR_CUDA;
+  }
   trace_mark(stream, "rollback.move");
   // cooperative (every CTA resident), and allowed to launch while the map
   // kernel finishes (the kernel waits for it before reading the plan)

@@ -19,7 +19,10 @@ def test_many_prompts_match_oracle(B, hi):
     lens[:5] = ([hi, 127, 128, 129, 64] if hi > 128 else [hi] * 5)[:B]
     lens[-1] = hi
     T = int(lens.sum())
-    q, k, v = (W.bf16_normal((T, h, 64), 1.0, 300 + B + h, dv) for h in (2, 1, 1))
+    # rows that see one to three keys return nearly v itself: with |v| < 2 (8 standard deviations) the output's
+    # bf16 rounding is at most 2^-8 and the fp16 operands add at most 2 * 2 * 2^-11, within the tolerance of 1e-2
+    # (with N(0, 1) values above 4 the rounding alone is 2^-6)
+    q, k, v = (W.bf16_normal((T, h, 64), std, 300 + B + h, dv) for h, std in ((2, 1.0), (1, 1.0), (1, 0.25)))
     cu = torch.tensor(np.concatenate([[0], np.cumsum(lens)]), dtype=torch.int32, device=dv)
     status = m.new_status(dv)
     out = m.umim_prefill_attention(q, k, v, cu, dev_status=status)

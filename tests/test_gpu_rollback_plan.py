@@ -16,6 +16,8 @@ pytestmark = pytest.mark.gpu
     ([17000], [8192], 1, 2), ([17000], [8193], 1, 2),                # one and two passes
     ([3000], [1], 2900, 2900),                                       # a span over many pages
     ([257, 0, 256, 255], [1, 0, 1, 1], 1, 1),
+    ([4096, 100], [4096, 100], 1, 1), ([4090, 1024, 1025], [1300, 7, 300], 2, 4),   # plan and map in one kernel: 256 pages
+    ([4097, 64], [1300, 20], 2, 4),                                                  # and in two: 257
 ])
 def test_span_counts_match_oracle(lens, n_spans, kmin, kmax):
     m = umim()
@@ -28,3 +30,19 @@ def test_span_counts_match_oracle(lens, n_spans, kmin, kmax):
     torch.cuda.synchronize()
     assert int(status.item()) == 0
     compare_rollback(g["pool"], g["bt"], g["lens"], freed, oracle_rollback(c))
+
+
+def test_more_spans_than_entries_are_refused():
+    """More spans than a 256-page table has entries: invalid, nothing written."""
+    m = umim()
+    c = W.decode_case(77, lens=[4096], n_q_heads=2, n_kv_heads=1, head_dim=64, n_spans=[0])
+    g = case_to_dev(c, dev())
+    S = 5000
+    i32 = lambda x: torch.as_tensor(x, dtype=torch.int32, device=dev())
+    sur = torch.zeros((S, 1, 1, 64), dtype=torch.bfloat16, device=dev())
+    status, before, table = m.new_status(dev()), g["pool"].clone(), g["bt"].clone()
+    m.umim_kv_rollback(g["pool"], g["bt"], g["lens"], i32([0, S]), i32(np.arange(S) % 4096), i32(np.ones(S)), sur, sur,
+                       dev_status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 1
+    assert torch.equal(g["pool"], before) and torch.equal(g["bt"], table) and int(g["lens"][0]) == 4096

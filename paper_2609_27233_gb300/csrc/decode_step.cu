@@ -40,6 +40,10 @@ constexpr int kStepWarps = 12;
 constexpr int kStepStages = 2;
 constexpr int kStepThreads = kStepWarps * 32;
 constexpr int kStepMaxBatch = 4096;
+// A split segment of more pieces is merged by all warps of its last CTA: two pieces
+// or more to a warp.  Below it a warp's own six rounds of four pieces cost about
+// as much as the parts' way through shared memory and the CTA's barriers.
+constexpr int kSharedPieces = 24;
 
 // workspace: a 256-byte header, per-segment arrival counters, then two partial
 // slots per warp (a warp's range meets at most two split segments: the one it
@@ -173,6 +177,7 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   __shared__ uint64_t bars[kStepWarps][kStepStages];
   __shared__ int s_scan[kStepWarps];
   __shared__ int s_last;
+  __shared__ int s_pend[kStepWarps][2];   // split segments this warp is to merge (-1: none)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gw = blockIdx.x * kStepWarps + warp;
@@ -182,6 +187,7 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   int *pref = reinterpret_cast<int *>(base + kStepWarps * kStepStages * kStage);   // [B + 1] units before b
 
   if (lane == 0) {
+    s_pend[warp][0] = s_pend[warp][1] = -1;
     for (int s = 0; s < kStepStages; ++s) mbar_init(&bars[warp][s], 1);
     fence_mbar_init();
     if (warp == 0) prefetch_tensormap(&kv_map);
@@ -326,7 +332,7 @@ __global__ void __launch_bounds__(kStepThreads, 1)
 
     // the current segment (cb, cg) is finished within this warp's range: write
     // its output, or its partial and, if this warp is the segment's last to
-    // finish, the merged output
+    // finish, note that the segment is this warp's to merge
     auto flush = [&]() {
       float s0 = l0, s1 = l1;
       s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
@@ -372,67 +378,7 @@ __global__ void __launch_bounds__(kStepThreads, 1)
       const int w0 = o / W, w1 = (o + n - 1) / W;
       if (old != w1 - w0) return;   // another warp of the segment is still running
       if (!in_bounds(w1, (int64_t)gridDim.x * kStepWarps, a.status, kSiteStepPartial)) return;
-      // last to finish: merge the segment's partials (warp w0 used slot 1
-      // unless the segment starts its range; every later warp used slot 0),
-      // several pieces' loads in flight at a time
-      __threadfence();
-      constexpr int U = E == 4 ? 4 : 8;
-      for (int r = 0; r < G; ++r) {
-        float M = -INFINITY, l = 0.f, ov[E];
-#pragma unroll
-        for (int e = 0; e < E; ++e) ov[e] = 0.f;
-        for (int w = w0; w <= w1; w += U) {
-          float2 pm[U];
-          float av[U][E];
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            pm[u] = make_float2(-INFINITY, 0.f);
-#pragma unroll
-            for (int e = 0; e < E; ++e) av[u][e] = 0.f;
-            if (w + u <= w1) {
-              const int sl = (w + u == w0 && o != w0 * W) ? 1 : 0;
-              const int64_t pc = ((int64_t)(w + u) * 2 + sl) * 16 + r;
-              pm[u] = __ldcg(ws.part_ml + pc);
-              if constexpr (E == 4) {
-                const float4 f = __ldcg(reinterpret_cast<const float4 *>(ws.part_acc + pc * D + lane * E));
-                av[u][0] = f.x, av[u][1] = f.y, av[u][2] = f.z, av[u][3] = f.w;
-              } else {
-                const float2 f = __ldcg(reinterpret_cast<const float2 *>(ws.part_acc + pc * D + lane * E));
-                av[u][0] = f.x, av[u][1] = f.y;
-              }
-            }
-          }
-          float nm = M;
-#pragma unroll
-          for (int u = 0; u < U; ++u) nm = fmaxf(nm, pm[u].x);
-          if (nm == -INFINITY) continue;
-          const float c_old = exp2f(M - nm);
-          l *= c_old;
-#pragma unroll
-          for (int e = 0; e < E; ++e) ov[e] *= c_old;
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const float c = exp2f(pm[u].x - nm);   // 0 for an absent or empty piece
-            l = fmaf(pm[u].y, c, l);
-#pragma unroll
-            for (int e = 0; e < E; ++e) ov[e] = fmaf(av[u][e], c, ov[e]);
-          }
-          M = nm;
-        }
-        const float inv = l > 0.f ? 1.f / l : 0.f;
-        if constexpr (E == 4) {
-          __nv_bfloat162 lo = __floats2bfloat162_rn(ov[0] * inv, ov[1] * inv);
-          __nv_bfloat162 hi = __floats2bfloat162_rn(ov[2] * inv, ov[3] * inv);
-          uint2 pk;
-          pk.x = *reinterpret_cast<uint32_t *>(&lo);
-          pk.y = *reinterpret_cast<uint32_t *>(&hi);
-          *reinterpret_cast<uint2 *>(obase + (int64_t)r * D + lane * E) = pk;
-        } else {
-          *reinterpret_cast<__nv_bfloat162 *>(obase + (int64_t)r * D + lane * E) =
-              __floats2bfloat162_rn(ov[0] * inv, ov[1] * inv);
-        }
-      }
-      if (lane == 0) ws.cnt[seg] = 0;   // ready for the next call
+      if (lane == 0) s_pend[warp][slot] = seg;   // last to finish: merged below
     };
 
     int it = 0;
@@ -594,6 +540,157 @@ __global__ void __launch_bounds__(kStepThreads, 1)
       }
     }
     (void)dead;
+  }
+
+  // ---- merge the segments that this CTA's warps were the last of (the one a
+  // warp's range starts in and the one it ends in, at most).  After the attention
+  // loop the registers of its queries and accumulators are free, so that four
+  // rows' and four pieces' loads are in flight together; row by row inside the
+  // loop, a segment of seven rows in 15 pieces waited for memory 28 times over,
+  // longer than its keys took.  A segment in many pieces (few, long sequences) is
+  // shared by the CTA's warps: each merges a part of the pieces, and the parts
+  // meet in the ring's shared memory.  A layer of 28/4 heads over 30 sequences
+  // (median 900): 64 -> 34 us; of 32/8 over one sequence of 8000: 81 -> 21; one
+  // warp's share of the latter without the CTA's help 40 ----
+  constexpr int U = 4, R = 4;
+  // rows r0 .. r0 + 3 of segment (b, g) over its pieces wa .. wb
+  auto merge_pieces = [&](int o, int wa, int wb, int r0, float (&M)[R], float (&l)[R], float (&ov)[R][E]) {
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      M[i] = -INFINITY;
+      l[i] = 0.f;
+#pragma unroll
+      for (int e = 0; e < E; ++e) ov[i][e] = 0.f;
+    }
+#pragma unroll 1
+    for (int w = wa; w <= wb; w += U) {
+      float2 pm[R][U];
+      float av[R][U][E];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        // the segment's first warp used slot 1 unless the segment starts its range, every later one slot 0
+        const int sl = w + u == o / W && o % W != 0 ? 1 : 0;
+        const int64_t piece = ((int64_t)(w + u) * 2 + sl) * 16 + r0;
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          pm[i][u] = make_float2(-INFINITY, 0.f);
+#pragma unroll
+          for (int e = 0; e < E; ++e) av[i][u][e] = 0.f;
+          if (w + u <= wb && r0 + i < G) {
+            const int64_t pc = piece + i;
+            pm[i][u] = __ldcg(ws.part_ml + pc);
+            if constexpr (E == 4) {
+              const float4 f = __ldcg(reinterpret_cast<const float4 *>(ws.part_acc + pc * D + lane * E));
+              av[i][u][0] = f.x, av[i][u][1] = f.y, av[i][u][2] = f.z, av[i][u][3] = f.w;
+            } else {
+              const float2 f = __ldcg(reinterpret_cast<const float2 *>(ws.part_acc + pc * D + lane * E));
+              av[i][u][0] = f.x, av[i][u][1] = f.y;
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        float nm = M[i];
+#pragma unroll
+        for (int u = 0; u < U; ++u) nm = fmaxf(nm, pm[i][u].x);
+        if (nm == -INFINITY) continue;
+        const float c_old = exp2f(M[i] - nm);
+        l[i] *= c_old;
+#pragma unroll
+        for (int e = 0; e < E; ++e) ov[i][e] *= c_old;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const float c = exp2f(pm[i][u].x - nm);   // 0 for an absent or empty piece
+          l[i] = fmaf(pm[i][u].y, c, l[i]);
+#pragma unroll
+          for (int e = 0; e < E; ++e) ov[i][e] = fmaf(av[i][u][e], c, ov[i][e]);
+        }
+        M[i] = nm;
+      }
+    }
+  };
+  auto write_row = [&](int seg, int r, float l, const float (&ov)[E]) {
+    const int b = seg / Hkv, g = seg - b * Hkv;
+    const float inv = l > 0.f ? 1.f / l : 0.f;
+    __nv_bfloat16 *orow = a.out + ((int64_t)b * a.Hq + (int64_t)g * G + r) * D + lane * E;
+#pragma unroll
+    for (int e = 0; e < E; e += 2)
+      *reinterpret_cast<__nv_bfloat162 *>(orow + e) = __floats2bfloat162_rn(ov[e] * inv, ov[e + 1] * inv);
+  };
+  struct Split {
+    int o, w0, w1;   // first unit, first and last warp
+  };
+  auto split_of = [&](int seg) {
+    const int b = seg / Hkv, g = seg - b * Hkv;
+    const int n = pref[b + 1] - pref[b], o = Hkv * pref[b] + g * n;
+    return Split{o, o / W, (o + n - 1) / W};
+  };
+  __syncwarp();
+  bool shared = false;
+  for (int slot = 0; slot < 2; ++slot) {
+    const int seg = s_pend[warp][slot];
+    if (seg < 0) continue;
+    const Split sp = split_of(seg);
+    if (sp.w1 - sp.w0 >= kSharedPieces) {
+      shared = true;   // left for the whole CTA
+      continue;
+    }
+    __threadfence();
+#pragma unroll 1
+    for (int r0 = 0; r0 < G; r0 += R) {
+      float M[R], l[R], ov[R][E];
+      merge_pieces(sp.o, sp.w0, sp.w1, r0, M, l, ov);
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+        if (r0 + i < G) write_row(seg, r0 + i, l[i], ov[i]);
+    }
+    __syncwarp();
+    if (lane == 0) {
+      ws.cnt[seg] = 0;   // ready for the next call
+      s_pend[warp][slot] = -1;
+    }
+  }
+  if (__syncthreads_or(shared)) {
+    __threadfence();
+    float *part = reinterpret_cast<float *>(base);   // [warps][16 rows][D], then (m, l) pairs
+    float2 *part_ml = reinterpret_cast<float2 *>(part + kStepWarps * 16 * D);
+    for (int k = 0; k < 2 * kStepWarps; ++k) {
+      const int seg = s_pend[k >> 1][k & 1];
+      if (seg < 0) continue;
+      const Split sp = split_of(seg);
+      const int per = (sp.w1 - sp.w0 + kStepWarps) / kStepWarps;
+      const int wa = sp.w0 + warp * per, wb = min(sp.w1, wa + per - 1);
+#pragma unroll 1
+      for (int r0 = 0; r0 < G; r0 += R) {
+        float M[R], l[R], ov[R][E];
+        merge_pieces(sp.o, wa, wb, r0, M, l, ov);
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+          if (r0 + i < G) {
+            if (lane == 0) part_ml[warp * 16 + r0 + i] = make_float2(M[i], l[i]);
+#pragma unroll
+            for (int e = 0; e < E; ++e) part[(warp * 16 + r0 + i) * D + lane * E + e] = ov[i][e];
+          }
+      }
+      __syncthreads();
+      for (int r = warp; r < G; r += kStepWarps) {
+        float M = -INFINITY, l = 0.f, ov[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) ov[e] = 0.f;
+        for (int w = 0; w < kStepWarps; ++w) M = fmaxf(M, part_ml[w * 16 + r].x);
+        for (int w = 0; w < kStepWarps && M != -INFINITY; ++w) {
+          const float2 ml = part_ml[w * 16 + r];
+          const float c = exp2f(ml.x - M);
+          l = fmaf(ml.y, c, l);
+#pragma unroll
+          for (int e = 0; e < E; ++e) ov[e] = fmaf(part[(w * 16 + r) * D + lane * E + e], c, ov[e]);
+        }
+        write_row(seg, r, l, ov);
+      }
+      if (threadIdx.x == 0) ws.cnt[seg] = 0;   // ready for the next call
+      __syncthreads();
+    }
   }
 
   // ---- commit (the step's last layer): once every CTA is done reading ----

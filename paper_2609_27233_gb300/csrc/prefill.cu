@@ -4,30 +4,30 @@
 // then runs over the shorter sequences).  Sequence b owns rows
 // cu_seqlens[b] .. cu_seqlens[b+1]-1 of q [T][Hq][D], k, v [T][Hkv][D].
 //
-// On the 5th-generation tensor cores, in one of two kernels: one head at a time,
-// described here, or two heads of an even group at a time (below), for enough work.
-// One head: a persistent kernel, two CTAs per SM (each allocates half of the tensor memory, so one CTA's products fill the
-// tensor cores while the other's softmax runs), each walking work units of
-// 128 query rows of one sequence for one query head, heaviest first; the
-// next unit's Q and K loads and first S products overlap the current unit's
-// last tiles and epilogue.  Warp 0 loads tiles with TMA (a unit's Q; 64-key K
-// tiles into a 2-stage ring running a tile ahead of the V^T tiles' 2-stage
-// ring), warp 1 issues the S = Q K^T products (tcgen05.mma into one of two
-// tensor-memory buffers, reused once the P V product that read it is done),
-// warp 6 the O += P V products into a tensor-memory accumulator (a separate
-// issuing thread, so that a P V product never waits behind an S product that
-// waits for the previous P V), and warps 2-5 run the online
-// softmax, one thread per query row: S from tensor memory (tcgen05.ld),
-// causal mask, running max, P = exp2(S - max) written back in fp16 over the
-// S columns it came from (tcgen05.st; the P V product reads its A operand
-// from tensor memory, so P never touches shared memory), row sums.  P V runs
-// on fp16 operands (V^T is converted when it is transposed): fp16's 11-bit
-// significand keeps P's and V's rounding near 3e-4 relative, where bf16 P
-// would cost 1e-3 of the output's error budget; P <= 2^8 by construction and
-// |v| < 65504 is checked (UMIM_ERR_UNSUPPORTED otherwise).  The running max
-// is only moved when it grows by more than 2^8, so the accumulator in tensor
-// memory is rescaled rarely (the result is the same: P and the row sum use
-// the same stale max).
+// On the 5th-generation tensor cores, in one of two kernels: one head at a
+// time, described here, or two heads of an even group at a time (below), for
+// enough work.  One head: a persistent kernel, two CTAs per SM (each allocates
+// half of the tensor memory, so one CTA's products fill the tensor cores while
+// the other's softmax runs), each walking work units of 128 query rows of one
+// sequence for one query head, heaviest first; the next unit's Q and K loads
+// and first S products overlap the current unit's last tiles and epilogue.
+// Warp 0 loads tiles with TMA (a unit's Q; 64-key K tiles into a 2-stage ring
+// running a tile ahead of the V^T tiles' 2-stage ring), warp 1 issues the S = Q
+// K^T products (tcgen05.mma into one of two tensor-memory buffers, reused once
+// the P V product that read it is done), warp 6 the O += P V products into a
+// tensor-memory accumulator (a separate issuing thread, so that a P V product
+// never waits behind an S product that waits for the previous P V), and warps
+// 2-5 run the online softmax, one thread per query row: S from tensor memory
+// (tcgen05.ld), causal mask, running max, P = exp2(S - max) written back in
+// fp16 over the S columns it came from (tcgen05.st; the P V product reads its A
+// operand from tensor memory, so P never touches shared memory), row sums.  P V
+// runs on fp16 operands (V^T is converted when it is transposed): fp16's 11-bit
+// significand keeps P's and V's rounding near 3e-4 relative, where bf16 P would
+// cost 1e-3 of the output's error budget; P <= 2^8 by construction and |v| <
+// 65504 is checked (UMIM_ERR_UNSUPPORTED otherwise).  The running max is only
+// moved when it grows by more than 2^8, so the accumulator in tensor memory is
+// rescaled rarely (the result is the same: P and the row sum use the same stale
+// max).
 //
 // V is transposed first (per sequence, padded to a multiple of 64 keys) so
 // that both products read K-major operands and every TMA copy starts on a

@@ -205,8 +205,8 @@ __global__ void __launch_bounds__(kMapThreads) rollback_map_kernel(MoveArgs a, P
 // table has at most kPlanMapPages columns: the spans stay in shared memory and
 // the block maps its pages, 64 a pass.  A kernel of its own for the map costs a
 // launch and the trips above, and pays once a sequence has many passes.
-// Plan and map of a 512-entry table's step, traced: 12.3 + 8.3 -> 12.5 us; of 16
-// sequences of 4096 entries: 12.5 + 9.4 -> 18.8 us.
+// Plan and map of a 512-entry table's step, traced: 12.3 + 8.3 -> 12.5 us (10.8
+// since one warp builds the totals); of 16 sequences of 4096 entries: 12.5 + 9.4 -> 18.8.
 constexpr int kPlanMapPages = 256;
 constexpr int kPlanMapSpans = kPlanMapPages * kPageSize;   // a span replaces an entry at least
 

@@ -577,6 +577,12 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
       if (k + S < my_units) next_unit(Nx);
     }
     if (!__all_sync(0xffffffffu, mbar_wait(&bars[wid][st], (uint32_t)(k / S) & 1u))) return false;
+    // the unit's rows are in shared memory, so its reads of the old pages are done: count it
+    // (relaxed: a release would also wait for this thread's earlier bulk stores to reach memory),
+    // before the rotation, which the units that wait for the count need not wait for (four
+    // sequences of 32768 entries, rollback with rotation and attention: 142.8 -> 141.3 us)
+    if (cur.valid && elect_one())
+      asm volatile("red.relaxed.gpu.global.add.s32 [%0], 1;" ::"l"(&pd.dep[cur.idx].landed) : "memory");
     if (ROPE && cur.valid && cur.kv == 0) {
       rotate_rows(cur, ring + st * TILE);
       fence_proxy_async_smem();   // the rotated rows, written by the lanes, are what the bulk store reads
@@ -584,9 +590,6 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
     }
     bool ok = true;
     if (cur.valid && elect_one()) {   // (the same lane every time: it waits for its own stores)
-      // the unit's rows are in shared memory, so its reads of the old pages are done: count it
-      // (relaxed: a release would also wait for this thread's earlier bulk stores to reach memory)
-      asm volatile("red.relaxed.gpu.global.add.s32 [%0], 1;" ::"l"(&pd.dep[cur.idx].landed) : "memory");
       ok = readers_done(cur);
       if (ok && cur.rb > cur.ra) {
         fence_proxy_async_global();

@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   __shared__ int s_last;
   __shared__ int s_pend[kStepWarps][2];   // split segments this warp is to merge (-1: none)
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int gw = blockIdx.x * kStepWarps + warp;
   const int total_warps = gridDim.x * kStepWarps;
   uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));

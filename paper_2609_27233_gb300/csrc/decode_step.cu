@@ -378,7 +378,7 @@ __global__ void __launch_bounds__(kStepThreads, 1)
       const int w0 = o / W, w1 = (o + n - 1) / W;
       if (old != w1 - w0) return;   // another warp of the segment is still running
       if (!in_bounds(w1, (int64_t)gridDim.x * kStepWarps, a.status, kSiteStepPartial)) return;
-      if (lane == 0) s_pend[warp][slot] = seg;   // last to finish: merged below
+      if (lane == 0) s_pend[warp][slot] = seg;   // last to finish: merged below (after a fence there)
     };
 
     int it = 0;
@@ -626,6 +626,12 @@ __global__ void __launch_bounds__(kStepThreads, 1)
     const int n = pref[b + 1] - pref[b], o = Hkv * pref[b] + g * n;
     return Split{o, o / W, (o + n - 1) / W};
   };
+  // The counts are relaxed.  Lane 0, which counted, fences once more after them:
+  // with the fence that each other warp made before it counted, that warp's
+  // partials come before this point, and the barriers below pass the order on to
+  // the lanes and warps that read them (their own fences could not: they counted
+  // nothing).
+  if (lane == 0 && (s_pend[warp][0] >= 0 || s_pend[warp][1] >= 0)) __threadfence();
   __syncwarp();
   bool shared = false;
   for (int slot = 0; slot < 2; ++slot) {
@@ -636,7 +642,6 @@ __global__ void __launch_bounds__(kStepThreads, 1)
       shared = true;   // left for the whole CTA
       continue;
     }
-    __threadfence();
 #pragma unroll 1
     for (int r0 = 0; r0 < G; r0 += R) {
       float M[R], l[R], ov[R][E];
@@ -652,7 +657,6 @@ __global__ void __launch_bounds__(kStepThreads, 1)
     }
   }
   if (__syncthreads_or(shared)) {
-    __threadfence();
     float *part = reinterpret_cast<float *>(base);   // [warps][16 rows][D], then (m, l) pairs
     float2 *part_ml = reinterpret_cast<float2 *>(part + kStepWarps * 16 * D);
     for (int k = 0; k < 2 * kStepWarps; ++k) {

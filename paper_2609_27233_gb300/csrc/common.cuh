@@ -110,6 +110,18 @@ __device__ __forceinline__ int32_t ld_acquire(const int32_t *p) {
   return v;
 }
 
+// Counts a CTA in at *cnt; true for the last of n.  One thread calls it, after a
+// barrier of its CTA.  The add is relaxed: the fence before it puts the CTA's
+// accesses before the count, the last caller's fence after it puts every other
+// CTA's accesses before what it does next.  A barrier then hands that order on to
+// the last CTA's other threads (their own fences could not: they counted nothing).
+__device__ __forceinline__ bool arrive_is_last(int32_t *cnt, int n) {
+  __threadfence();
+  const bool last = atomicAdd(cnt, 1) == n - 1;
+  if (last) __threadfence();
+  return last;
+}
+
 // ---------------------------------------------------------------------------
 // mbarrier
 // ---------------------------------------------------------------------------

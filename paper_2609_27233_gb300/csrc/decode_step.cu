@@ -701,12 +701,10 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   if (a.commit) {
     __syncthreads();
     if (threadIdx.x == 0) {
-      __threadfence();
-      s_last = atomicAdd(&ws.hdr->done, 1) == (int)gridDim.x - 1;
+      s_last = arrive_is_last(&ws.hdr->done, (int)gridDim.x);
     }
     __syncthreads();
     if (s_last) {
-      __threadfence();
       for (int b = threadIdx.x; b < B; b += kStepThreads) {
         const SeqStep st = seq_step(a, b);
         if (st.slot < 0) {

@@ -179,13 +179,11 @@ __global__ void __launch_bounds__(kAlignThreads) align_plan_kernel(AlignArgs a, 
     arr.Lc[b] = Lc;
     arr.first[b] = (!err && hi > lo) ? a.span_start[lo] : Lc;
     if (err) atomicOr(&arr.hdr->error, 1);
-    __threadfence();
-    s_last = atomicAdd(&arr.hdr->blocks_done, 1) == (int)gridDim.x - 1;
+    s_last = arrive_is_last(&arr.hdr->blocks_done, (int)gridDim.x);
   }
   __syncthreads();
   if (!s_last) return;
 
-  __threadfence();
   int err = atomicOr(&arr.hdr->error, 0);
   long long ct = 0, cs = 0, cp = 0;
   for (int base = 0; base < a.B; base += kAlignThreads) {
@@ -823,12 +821,10 @@ __global__ void __launch_bounds__(T + 32, 1) ce_kernel(CeArgs a) {
   __shared__ int s_last;
   __syncthreads();
   if (tid == 0) {
-    __threadfence();
-    s_last = atomicAdd(&a.hdr->ctas_done, 1) == (int)gridDim.x - 1;
+    s_last = arrive_is_last(&a.hdr->ctas_done, (int)gridDim.x);
   }
   __syncthreads();
   if (!s_last) return;
-  __threadfence();
   __shared__ double dpart[NW + 1];
   const int per = (N + NT - 1) / NT;
   double acc = 0.0;

@@ -169,9 +169,7 @@ __device__ inline PlanSeq plan_sequence(const PlanArgs &a, const PlanArrays &arr
     arr.first_page[b] = fp;
     arr.n_dest[b] = nd;
     if (err) atomicOr(&arr.hdr->error, 1);
-    __threadfence();
-    const int done = atomicAdd(&arr.hdr->blocks_done, 1);
-    s_last = (done == (int)gridDim.x - 1);
+    s_last = arrive_is_last(&arr.hdr->blocks_done, (int)gridDim.x);
   }
   __syncthreads();
   return {L, Lp, lo, hi, fp, nd, s_last != 0};
@@ -209,7 +207,6 @@ constexpr int kTotItems = 4;
 
 __device__ inline void plan_totals_warp(const PlanArgs &a, const PlanArrays &arr) {
   const int lane = threadIdx.x & 31;
-  __threadfence();
   int err = lane == 0 ? atomicOr(&arr.hdr->error, 0) : 0;
   const int32_t epoch = lane == 0 ? __ldcg(&arr.hdr->epoch) : 0;
   int L[kTotItems], Lp[kTotItems], nd[kTotItems];
@@ -269,7 +266,6 @@ __device__ inline void plan_totals(const PlanArgs &a, const PlanArrays &arr) {
     if (threadIdx.x < 32) plan_totals_warp(a, arr);
     return;
   }
-  __threadfence();
   const int err = atomicOr(&arr.hdr->error, 0);
   int cu_units = 0, cu_rows = 0, cu_freed = 0, cu_active = 0;
   __shared__ int s_max_dest;

@@ -232,13 +232,10 @@ __device__ void finish_rollback(const MoveArgs &a, const PlanArrays &arr, int &s
   const int tid = threadIdx.x;
   __syncthreads();
   if (tid == 0) {
-    __threadfence();
-    const int done = atomicAdd(&arr.hdr->done_ctas, 1);
-    s_last = (done == (int)gridDim.x - 1);
+    s_last = arrive_is_last(&arr.hdr->done_ctas, (int)gridDim.x);
   }
   __syncthreads();
   if (!s_last || arr.hdr->skip) return;
-  __threadfence();
   for (int b = 0; b < a.B; ++b) {
     if (a.span_offsets[b + 1] == a.span_offsets[b]) continue;
     const int L = arr.seq_L[b], Lp = arr.seq_Lp[b];

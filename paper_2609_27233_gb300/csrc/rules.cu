@@ -412,12 +412,10 @@ __global__ void __launch_bounds__(kWalkThreads) prompt_walk_kernel(MatchArgs a, 
   // the last CTA: span and token offsets of every prompt
   __syncthreads();
   if (tid == 0) {
-    __threadfence();
-    s_last = atomicAdd(&w.hdr->done, 1) == a.B - 1;
+    s_last = arrive_is_last(&w.hdr->done, a.B);
   }
   __syncthreads();
   if (!s_last) return;
-  __threadfence();
   int cs = 0, ct = 0;
   for (int base = 0; base < a.B; base += kWalkThreads) {
     const int i = base + tid;

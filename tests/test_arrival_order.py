@@ -21,3 +21,24 @@ def test_layer_step_fences_between_its_counts_and_the_merge():
     assert fence, "lane 0 counts: it fences, then the warp's barrier hands the partials on"
     # and the CTA's barrier stands between that fence and the merges that all warps share
     assert code.index("__syncthreads_or(shared)", counted) < code.index("merge_pieces(sp.o, wa", counted)
+
+
+def test_last_ctas_fence_before_their_barrier():
+    """Every count of CTAs goes through the helper that fences on both sides, and a CTA's barrier follows it; the only
+    other add to a counter in global memory is the layer step's (above)."""
+    helper = _code("common.cuh")
+    body = helper[helper.index("bool arrive_is_last("):]
+    body = body[:body.index("\n}")]
+    assert re.search(r"__threadfence\(\);.*atomicAdd\(.*if \(last\) __threadfence\(\);", body, flags=re.S)
+    calls = 0
+    for name in sorted(os.listdir(CSRC)):
+        code = _code(name)
+        for add in re.finditer(r"atomicAdd\(([^,]*),", code):
+            at = add.group(1).strip()
+            assert at.startswith("&s_") or (name, at) in (("common.cuh", "cnt"), ("decode_step.cu", "&ws.cnt[seg]")), \
+                (name, at)   # &s_...: shared memory
+        for call in re.finditer(r"= arrive_is_last\([^;]*\);\s*\}\s*(\w+\(\);)", code):
+            assert call.group(1) == "__syncthreads();", name
+            calls += 1
+        assert code.count("= arrive_is_last(") == len(re.findall(r"= arrive_is_last\([^;]*\);\s*\}\s*__syncthreads", code))
+    assert calls == 6

@@ -596,11 +596,10 @@ static umim_status run_attention(const void *q, int Hq, const umim_paged_kv *kv,
   a.n_layers = kv->n_layers;
   a.scale_log2 = scale * 1.4426950408889634f;
   a.status = status;
-  const size_t smem = (size_t)kAttnWarps * kAttnStages * 2 * 16 * D * 2 + 1024 +
-                      (smem_plan ? sizeof(int32_t) * ((size_t)B + 1) : 0);
+  constexpr size_t kRings = (size_t)kAttnWarps * kAttnStages * 2 * 16 * D * 2 + 1024;
+  const size_t smem = kRings + (smem_plan ? sizeof(int32_t) * ((size_t)B + 1) : 0);
   auto kern = attn_decode_kernel<D>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return UMIM_ERR_CUDA;
+  if (!allow_smem(kern, kRings + sizeof(int32_t) * (kSmemPlanBatch + 1))) return UMIM_ERR_CUDA;
   trace_mark(stream, "attention.decode");
   if (launch_pdl(kern, dim3(total_warps / kAttnWarps), dim3(kAttnWarps * 32), smem, stream, map, a, ws) !=
       cudaSuccess)

@@ -410,6 +410,16 @@ __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wa
 // this call is there for a kernel that reads it ahead of its own griddep_wait().
 __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Allows a kernel `most` bytes of dynamic shared memory.  The limit is one value per
+// function and device, which calls from other host threads set too: `most` is the
+// largest size that any call launches the function with, never this call's own size
+// (a smaller one, set by another thread between this and the launch, would refuse it).
+// Set on every call: the attribute belongs to the current device.
+template <typename Kern>
+inline bool allow_smem(Kern kern, size_t most) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) == cudaSuccess;
+}
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, unsigned cluster, size_t smem,
                                       cudaStream_t stream, Args... args) {

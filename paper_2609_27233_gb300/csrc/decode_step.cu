@@ -765,10 +765,10 @@ static umim_status run_step(const StepArgs &a0, const umim_paged_kv *kv, void *w
     return UMIM_ERR_CUDA;
   const int grid = std::max(1, num_sms);
   const StepWs ws = step_carve(workspace, a0.B, a0.Hkv, D, grid * kStepWarps);
-  const size_t smem = (size_t)kStepWarps * kStepStages * 2 * 16 * D * 2 + 1024 + sizeof(int32_t) * (a0.B + 1);
+  constexpr size_t kRings = (size_t)kStepWarps * kStepStages * 2 * 16 * D * 2 + 1024;
+  const size_t smem = kRings + sizeof(int32_t) * (a0.B + 1);
   auto kern = decode_step_kernel<D>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return UMIM_ERR_CUDA;
+  if (!allow_smem(kern, kRings + sizeof(int32_t) * (kStepMaxBatch + 1))) return UMIM_ERR_CUDA;
   trace_mark(stream, a0.commit ? "decode_step.commit" : "decode_step.layer");
   if (launch_pdl(kern, dim3(grid), dim3(kStepThreads), smem, stream, map, a0, ws) != cudaSuccess)
     return UMIM_ERR_CUDA;

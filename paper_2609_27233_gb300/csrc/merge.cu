@@ -23,6 +23,7 @@ namespace umim {
 namespace {
 
 constexpr int BM = 128, BN = 256, BK = 64, STAGES = 4;
+constexpr int kMaxWidth = 8192;   // the widest d_model that umim_merge_spans takes
 constexpr int kGemmThreads = 224;   // warp 0: TMA, warp 1: MMA + TMEM owner, warps 2-5: epilogue, warp 6: side job
 constexpr int kStageBytes = (BM + BN) * BK * 2;
 constexpr int kGemmSmem = STAGES * kStageBytes + 1024;
@@ -1330,10 +1331,7 @@ static umim_status launch_gemm(EncodeTiledFn enc, const void *A, const void *Bw,
   g.K = d;
   g.idesc = idesc_f32acc(BM, BN, fp16);
   auto kern = split > 1 ? (fp16 ? gemm_splitk_kernel<true> : gemm_splitk_kernel<false>) : gemm_bias_gelu_kernel;
-  // set on every call: the attribute belongs to the current device, and calls may
-  // come for several devices and from several threads
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem) != cudaSuccess)
-    return UMIM_ERR_CUDA;
+  if (!allow_smem(kern, kGemmSmem)) return UMIM_ERR_CUDA;
   trace_mark(st, label);
   return launch_pdl_cluster(kern, dim3(gemm_grid(g.M, d, num_sms)), dim3(split > 1 ? kSkThreads : kGemmThreads),
                             (unsigned)split, kGemmSmem, st, am, bm, g) == cudaSuccess
@@ -1421,8 +1419,8 @@ umim_status merge_spans(const void *embeddings, int64_t vocab, const int32_t *to
         return UMIM_ERR_CUDA;
     }
     const int psmem = kHeadWarps * kHeadBufs * head_buf_bytes(dh, nt);
-    if (cudaFuncSetAttribute(pk, cudaFuncAttributeMaxDynamicSharedMemorySize, psmem) != cudaSuccess)
-      return UMIM_ERR_CUDA;
+    // (pool_head_kernel<cpl> takes heads of up to 256 cpl columns)
+    if (!allow_smem(pk, kHeadWarps * kHeadBufs * head_buf_bytes(256 * cpl, kMaxWidth / BN))) return UMIM_ERR_CUDA;
     // warps of the grid: a multiple of h, at most one CTA per SM and no more than the items
     const int h = w->n_heads;
     const int64_t items = (int64_t)S * h;
@@ -1439,8 +1437,7 @@ umim_status merge_spans(const void *embeddings, int64_t vocab, const int32_t *to
     const int psmem = kPoolRing * pool_stage_bytes(d);
     const int chunks = d / 8 / kPoolConsumers;   // 16-byte column chunks per consumer thread (d <= 8192)
     auto pk = chunks <= 1 ? pool_kernel<1> : (chunks == 2 ? pool_kernel<2> : pool_kernel<4>);
-    if (cudaFuncSetAttribute(pk, cudaFuncAttributeMaxDynamicSharedMemorySize, psmem) != cudaSuccess)
-      return UMIM_ERR_CUDA;
+    if (!allow_smem(pk, kPoolRing * pool_stage_bytes(kMaxWidth))) return UMIM_ERR_CUDA;
     int pool_per_sm = 1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pool_per_sm, pk, kPoolConsumers + 32, psmem) != cudaSuccess ||
         pool_per_sm < 1)

@@ -1236,8 +1236,7 @@ umim_status prefill_attention(const void *q, const void *k, const void *v, int T
     if (!encode_3d(enc, &om, out, D, Hq, T, (uint64_t)D * 2, (uint64_t)Hq * D * 2, 64, 1, 32)) return UMIM_ERR_CUDA;
     auto kern = D == 128 ? prefill_pair_kernel<128> : prefill_pair_kernel<64>;
     const size_t smem = (size_t)(D == 128 ? PpSmem<128>::kTotal : PpSmem<64>::kTotal) + 1024;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return UMIM_ERR_CUDA;
+    if (!allow_smem(kern, smem)) return UMIM_ERR_CUDA;
     trace_mark(stream, "prefill.attention");
     if (launch_pdl(kern, dim3((unsigned)sms), dim3(kPpThreads), smem, stream, qm, km, vm, om, a) != cudaSuccess)
       return UMIM_ERR_CUDA;
@@ -1246,8 +1245,7 @@ umim_status prefill_attention(const void *q, const void *k, const void *v, int T
   }
   auto kern = D == 128 ? prefill_tc_kernel<128> : prefill_tc_kernel<64>;
   const size_t smem = (size_t)(D == 128 ? PfSmem<128>::kTotal : PfSmem<64>::kTotal) + 1024;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return UMIM_ERR_CUDA;
+  if (!allow_smem(kern, smem)) return UMIM_ERR_CUDA;
   // persistent: two CTAs per SM walk the (query tile, head) units; no more
   // CTAs than an upper bound of the units (each sequence wastes less than one tile)
   const int64_t units_max = ((int64_t)(T + kPfRows - 1) / kPfRows + B) * Hq;

@@ -687,18 +687,14 @@ umim_status kv_rollback(const umim_paged_kv *kv, int32_t *block_table, int32_t m
                    : (D == 128 ? rollback_bulk_kernel<128, false> : rollback_bulk_kernel<64, false>);
   const int threads = kBulkThreads;
   const int smem = kBulkMovers * kBulkStages * kPageSize * D * 2;
-  // set on every call: the attribute belongs to the current device
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-    return UMIM_ERR_CUDA;
+  if (!allow_smem(kern, smem)) return UMIM_ERR_CUDA;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1)
     per_sm = 1;
   const int grid = std::max(1, num_sms) * per_sm;   // every CTA resident (cooperative launch)
   if (max_pages <= kPlanMapPages) {
     const int plan_smem = 4 * kPlanMapSpans * (int)sizeof(int32_t);
-    if (cudaFuncSetAttribute(rollback_plan_map_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, plan_smem) !=
-        cudaSuccess)
-      return UMIM_ERR_CUDA;
+    if (!allow_smem(rollback_plan_map_kernel, plan_smem)) return UMIM_ERR_CUDA;
     trace_mark(stream, "rollback.plan_map");
     if (launch_pdl(rollback_plan_map_kernel, dim3((unsigned)B), dim3(kPlanThreads), (size_t)plan_smem, stream, pa, ma,
                    arr, pd, (int)D) != cudaSuccess)

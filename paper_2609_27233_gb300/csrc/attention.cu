@@ -373,10 +373,12 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 1)
     mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
     mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
     mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
-    const float n0 = fmaxf(m0, mx0), n1 = fmaxf(m1, mx1);
-    const float c0 = exp2f(m0 - n0), c1 = exp2f(m1 - n1);
-    m0 = n0;
-    m1 = n1;
+    const float was0 = m0, was1 = m1;
+    m0 = fmaxf(m0, mx0);
+    m1 = fmaxf(m1, mx1);
+    // no finite score so far: weights from 0, so that a score of -inf weighs 0 and NaN stays NaN
+    const float n0 = m0 == -INFINITY ? 0.f : m0, n1 = m1 == -INFINITY ? 0.f : m1;
+    const float c0 = exp2f(was0 - n0), c1 = exp2f(was1 - n1);
     float p[2][4];
 #pragma unroll
     for (int nt = 0; nt < 2; ++nt) {
@@ -486,14 +488,15 @@ __global__ void __launch_bounds__(kCombineThreads)
     float nm = M;
 #pragma unroll
     for (int u = 0; u < U; ++u) nm = fmaxf(nm, ml[u].x);
-    if (nm == -INFINITY) continue;   // nothing but empty pieces so far
-    const float c_old = exp2f(M - nm);
+    // (a piece whose scores are all NaN has no maximum either, but a NaN sum: weighted, not skipped)
+    const float from = nm == -INFINITY ? 0.f : nm;
+    const float c_old = exp2f(M - from);
     l *= c_old;
 #pragma unroll
     for (int e = 0; e < E; ++e) o[e] *= c_old;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const float c = exp2f(ml[u].x - nm);   // 0 for an absent or empty piece
+      const float c = exp2f(ml[u].x - from);   // 0 for an absent or empty piece
       l = fmaf(ml[u].y, c, l);
 #pragma unroll
       for (int e = 0; e < E; ++e) o[e] = fmaf(av[u][e], c, o[e]);
@@ -515,19 +518,17 @@ __global__ void __launch_bounds__(kCombineThreads)
     l = 0.f;
 #pragma unroll
     for (int e = 0; e < E; ++e) o[e] = 0.f;
-    if (Mx != -INFINITY) {
+    if (Mx == -INFINITY) Mx = 0.f;
 #pragma unroll
-      for (int w = 0; w < WPR; ++w) {
-        if (s_m[warp + w] == -INFINITY) continue;
-        const float c = exp2f(s_m[warp + w] - Mx);
-        l += c * s_l[warp + w];
+    for (int w = 0; w < WPR; ++w) {
+      const float c = exp2f(s_m[warp + w] - Mx);
+      l += c * s_l[warp + w];
 #pragma unroll
-        for (int e = 0; e < E; ++e) o[e] += c * s_acc[warp + w][lane * E + e];
-      }
+      for (int e = 0; e < E; ++e) o[e] += c * s_acc[warp + w][lane * E + e];
     }
   }
   if (!live) return;
-  const float inv = l > 0.f ? 1.f / l : 0.f;
+  const float inv = p1 > p0 ? 1.f / l : 0.f;   // (no entries: zeros)
   __nv_bfloat16 *dst = out + ((int64_t)b * Hq + h) * D + lane * E;
 #pragma unroll
   for (int e = 0; e < E; ++e) dst[e] = __float2bfloat16_rn(o[e] * inv);

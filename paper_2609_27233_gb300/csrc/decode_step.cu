@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(kStepThreads, 1)
       const int o = Hkv * pref[cb] + cg * n;
       __nv_bfloat16 *obase = a.out + ((int64_t)cb * a.Hq + (int64_t)cg * G) * D;
       if (o >= start && o + n <= end) {
-        const float i0 = s0 > 0.f ? 1.f / s0 : 0.f, i1 = s1 > 0.f ? 1.f / s1 : 0.f;
+        const float i0 = 1.f / s0, i1 = 1.f / s1;
 #pragma unroll
         for (int j = 0; j < NT; ++j) {
           const int col = j * 8 + 2 * qc;
@@ -469,10 +469,12 @@ __global__ void __launch_bounds__(kStepThreads, 1)
       mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
       mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
       mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
-      const float n0 = fmaxf(m0, mx0), n1 = fmaxf(m1, mx1);
-      const float c0 = exp2f(m0 - n0), c1 = exp2f(m1 - n1);
-      m0 = n0;
-      m1 = n1;
+      const float was0 = m0, was1 = m1;
+      m0 = fmaxf(m0, mx0);
+      m1 = fmaxf(m1, mx1);
+      // no finite score so far: weights from 0, so that a score of -inf weighs 0 and NaN stays NaN
+      const float n0 = m0 == -INFINITY ? 0.f : m0, n1 = m1 == -INFINITY ? 0.f : m1;
+      const float c0 = exp2f(was0 - n0), c1 = exp2f(was1 - n1);
       float p[2][4];
 #pragma unroll
       for (int nt = 0; nt < 2; ++nt) {
@@ -553,7 +555,9 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   // (median 900): 64 -> 34 us; of 32/8 over one sequence of 8000: 81 -> 21; one
   // warp's share of the latter without the CTA's help 40 ----
   constexpr int U = 4, R = 4;
-  // rows r0 .. r0 + 3 of segment (b, g) over its pieces wa .. wb
+  // rows r0 .. r0 + 3 of segment (b, g) over its pieces wa .. wb.  A piece whose
+  // scores are all NaN has no maximum (-inf) but a NaN sum: pieces without one are
+  // weighted from 0, so that it reaches the output, not skipped as empty
   auto merge_pieces = [&](int o, int wa, int wb, int r0, float (&M)[R], float (&l)[R], float (&ov)[R][E]) {
 #pragma unroll
     for (int i = 0; i < R; ++i) {
@@ -594,14 +598,14 @@ __global__ void __launch_bounds__(kStepThreads, 1)
         float nm = M[i];
 #pragma unroll
         for (int u = 0; u < U; ++u) nm = fmaxf(nm, pm[i][u].x);
-        if (nm == -INFINITY) continue;
-        const float c_old = exp2f(M[i] - nm);
+        const float from = nm == -INFINITY ? 0.f : nm;
+        const float c_old = exp2f(M[i] - from);
         l[i] *= c_old;
 #pragma unroll
         for (int e = 0; e < E; ++e) ov[i][e] *= c_old;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const float c = exp2f(pm[i][u].x - nm);   // 0 for an absent or empty piece
+          const float c = exp2f(pm[i][u].x - from);   // 0 for an absent or empty piece, and 0 * NaN is NaN
           l[i] = fmaf(pm[i][u].y, c, l[i]);
 #pragma unroll
           for (int e = 0; e < E; ++e) ov[i][e] = fmaf(av[i][u][e], c, ov[i][e]);
@@ -612,7 +616,7 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   };
   auto write_row = [&](int seg, int r, float l, const float (&ov)[E]) {
     const int b = seg / Hkv, g = seg - b * Hkv;
-    const float inv = l > 0.f ? 1.f / l : 0.f;
+    const float inv = 1.f / l;
     __nv_bfloat16 *orow = a.out + ((int64_t)b * a.Hq + (int64_t)g * G + r) * D + lane * E;
 #pragma unroll
     for (int e = 0; e < E; e += 2)
@@ -683,7 +687,8 @@ __global__ void __launch_bounds__(kStepThreads, 1)
 #pragma unroll
         for (int e = 0; e < E; ++e) ov[e] = 0.f;
         for (int w = 0; w < kStepWarps; ++w) M = fmaxf(M, part_ml[w * 16 + r].x);
-        for (int w = 0; w < kStepWarps && M != -INFINITY; ++w) {
+        if (M == -INFINITY) M = 0.f;
+        for (int w = 0; w < kStepWarps; ++w) {
           const float2 ml = part_ml[w * 16 + r];
           const float c = exp2f(ml.x - M);
           l = fmaf(ml.y, c, l);

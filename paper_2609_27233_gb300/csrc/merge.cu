@@ -1435,7 +1435,7 @@ umim_status merge_spans(const void *embeddings, int64_t vocab, const int32_t *to
   } else {
     // wider heads: the CTA-per-span kernel with a staged ring
     const int psmem = kPoolRing * pool_stage_bytes(d);
-    const int chunks = d / 8 / kPoolConsumers;   // 16-byte column chunks per consumer thread (d <= 8192)
+    const int chunks = ceil_div(d / 8, kPoolConsumers);   // 16-byte column chunks per consumer thread (at most 4)
     auto pk = chunks <= 1 ? pool_kernel<1> : (chunks == 2 ? pool_kernel<2> : pool_kernel<4>);
     if (!allow_smem(pk, kPoolRing * pool_stage_bytes(kMaxWidth))) return UMIM_ERR_CUDA;
     int pool_per_sm = 1;

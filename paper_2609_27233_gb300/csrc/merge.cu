@@ -1301,15 +1301,20 @@ static bool encode_kmajor(EncodeTiledFn enc, CUtensorMap *map, const void *base,
 }
 
 // CTAs that share one tile's K range: as many as keep all clusters resident at
-// once (clusters of 8 leave some SMs of a GPC without a place: 7/8 of the SMs
-// are counted on), else 1.  A product whose tiles alone fill more than half of
-// that (one prompt's 714 tokens at d = 4096: 96 tiles) gains nothing from two
-// half-length waves.
+// once, else 1.  SMs of a GPC that do not make up a cluster stay empty: 152 SMs
+// hold 15 clusters of eight (36 of four, 76 of two), so 4/5 of the SMs are counted
+// on for eight and 7/8 for four and two.  A sixteenth cluster of eight is a second
+// wave: 1000 spans at d = 512 took 43.8 us so (in four 37.5), 128 at d = 4096
+// 61.6 (54.3).  A product whose tiles alone fill more than half of the SMs (one
+// prompt's 714 tokens at d = 4096: 96 tiles) gains nothing from two half-length
+// waves.
 static int gemm_split(int64_t M, int d, int num_sms) {
   const int64_t tiles = (int64_t)(d / BN) * ((M + BM - 1) / BM);
-  const int most = std::min(kFlagCtas, std::max(1, num_sms)) / 8 * 7;
-  for (int split = kSkMaxSplit; split > 1; split /= 2)
+  const int sms = std::min(kFlagCtas, std::max(1, num_sms));
+  for (int split = kSkMaxSplit; split > 1; split /= 2) {
+    const int most = split == 8 ? sms / 5 * 4 : sms / 8 * 7;
     if (tiles * split <= most && d / BK % split == 0) return split;
+  }
   return 1;
 }
 

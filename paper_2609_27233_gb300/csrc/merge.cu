@@ -1318,18 +1318,17 @@ static int gemm_split(int64_t M, int d, int num_sms) {
   return 1;
 }
 
-// CTAs of a product with M rows
-static int gemm_grid(int64_t M, int d, int num_sms) {
+// CTAs of a product with M rows, each tile's K range split over `split` of them
+static int gemm_grid(int64_t M, int d, int split, int num_sms) {
   const int64_t tiles = (int64_t)(d / BN) * ((M + BM - 1) / BM);
-  const int split = gemm_split(M, d, num_sms);
   return split > 1 ? (int)tiles * split : (int)std::min<int64_t>(tiles, std::min(kFlagCtas, std::max(1, num_sms)));
 }
 
 // out[M][d] = GELU(A[M][d] B[d][d]^T + bias).  A and B both bf16, or A fp16 and B
-// fp16 (bf16 when the product is split: gemm_split > 1).
-static umim_status launch_gemm(EncodeTiledFn enc, const void *A, const void *Bw, bool fp16, GemmArgs g,
+// fp16 (bf16 when the product is split).
+static umim_status launch_gemm(EncodeTiledFn enc, const void *A, const void *Bw, bool fp16, GemmArgs g, int split,
                                cudaStream_t st, const char *label, int num_sms) {
-  const int d = g.N, split = gemm_split(g.M, d, num_sms);
+  const int d = g.N;
   CUtensorMap am, bm;
   if (!encode_kmajor(enc, &am, A, g.M, d, BM, fp16) || !encode_kmajor(enc, &bm, Bw, d, d, BN, fp16 && split == 1))
     return UMIM_ERR_CUDA;
@@ -1338,7 +1337,7 @@ static umim_status launch_gemm(EncodeTiledFn enc, const void *A, const void *Bw,
   auto kern = split > 1 ? (fp16 ? gemm_splitk_kernel<true> : gemm_splitk_kernel<false>) : gemm_bias_gelu_kernel;
   if (!allow_smem(kern, kGemmSmem)) return UMIM_ERR_CUDA;
   trace_mark(st, label);
-  return launch_pdl_cluster(kern, dim3(gemm_grid(g.M, d, num_sms)), dim3(split > 1 ? kSkThreads : kGemmThreads),
+  return launch_pdl_cluster(kern, dim3(gemm_grid(g.M, d, split, num_sms)), dim3(split > 1 ? kSkThreads : kGemmThreads),
                             (unsigned)split, kGemmSmem, st, am, bm, g) == cudaSuccess
              ? UMIM_OK
              : UMIM_ERR_CUDA;
@@ -1372,15 +1371,21 @@ umim_status merge_spans(const void *embeddings, int64_t vocab, const int32_t *to
   };
 
   if (S == 0) return UMIM_OK;
-  // W_o -> fp16: inside a split output projection; else in a side warp of GEMM1
-  // when its share is small next to the tiles its CTA computes; else in a kernel
-  // of its own
-  const int grid1 = gemm_grid(T, d, num_sms);
+  // W_o -> fp16: inside a split output projection; else in a side warp of an
+  // unsplit GEMM1 when its share is small next to the tiles its CTA computes; else
+  // in a kernel of its own.  Where the side warp can take it, an output projection
+  // split no further than in two is not split at all: half a K loop costs more with
+  // the conversion in it and the exchange after it (2100 spans of 2 to 4 tokens at
+  // d = 512 44.2 us unsplit, 47.0 split, 1100 at d = 1024 45.8 and 48.1, 700 at
+  // d = 2048 56.2 and 57.9; without the side warp 450 at d = 3072 76.6 and 67.5)
+  const int split1 = gemm_split(T, d, num_sms);
+  const int grid1 = gemm_grid(T, d, split1, num_sms);
   const int64_t tiles1 = (int64_t)(d / BN) * ((T + BM - 1) / BM);
   const int64_t n_vec = (int64_t)d * d / 8;
-  const bool wo_split = gemm_split(S, d, num_sms) > 1;
-  const bool wo_in_gemm1 =
-      !wo_split && gemm_split(T, d, num_sms) == 1 && n_vec <= 128LL * 32 * grid1 * (tiles1 / grid1);
+  const bool side_warp = split1 == 1 && n_vec <= 128LL * 32 * grid1 * (tiles1 / grid1);
+  int split2 = gemm_split(S, d, num_sms);
+  if (split2 == 2 && side_warp) split2 = 1;
+  const bool wo_split = split2 > 1, wo_in_gemm1 = !wo_split && side_warp;
   GemmArgs g1{};
   g1.M = (int)T;
   g1.N = d;
@@ -1398,9 +1403,9 @@ umim_status merge_spans(const void *embeddings, int64_t vocab, const int32_t *to
   trace_mark(st, "merge.gather");
   if (launch_pdl(gather_rows_kernel, dim3(blocks), dim3(256), 0, st, static_cast<const uint4 *>(embeddings), vocab,
                  token_ids, T, d, reinterpret_cast<uint4 *>(E), status,
-                 gemm_split(T, d, num_sms) > 1 ? 1 : 0) != cudaSuccess)
+                 split1 > 1 ? 1 : 0) != cudaSuccess)
     return UMIM_ERR_CUDA;
-  umim_status r = launch_gemm(enc, E, w->w_kv, false, g1, st, "merge.gemm1", num_sms);
+  umim_status r = launch_gemm(enc, E, w->w_kv, false, g1, split1, st, "merge.gemm1", num_sms);
   if (r != UMIM_OK) return r;
   trace_mark(st, "merge.pool");
   const int Ch = d / w->n_heads / 8;   // 16-byte chunks per head
@@ -1470,10 +1475,10 @@ umim_status merge_spans(const void *embeddings, int64_t vocab, const int32_t *to
   g2.stats = st2;
   g2.acc_scale = 1.f / kWoScale;
   g2.prior = flags;
-  const int grid2 = gemm_grid(S, d, num_sms);
+  const int grid2 = gemm_grid(S, d, split2, num_sms);
   g2.range_flag = flag_words(kFlagGemm2, grid2);
   g2.status = status;
-  r = launch_gemm(enc, O, wo_split ? w->w_o : Wo16, true, g2, st, "merge.gemm2", num_sms);
+  r = launch_gemm(enc, O, wo_split ? w->w_o : Wo16, true, g2, split2, st, "merge.gemm2", num_sms);
   if (r != UMIM_OK) return r;
   trace_mark(st, "merge.ln_o");
   if (launch_pdl(ln_rows_kernel, dim3(std::min<int64_t>(S, (int64_t)std::max(1, num_sms) * (1536 / (d / 16)))),

@@ -56,3 +56,15 @@ def test_clusters_of_eight_fit_at_once(d, more):
     ran = check(case)
     for g in ("gemm1", "gemm2"):
         assert ran[g] == tiles(rows * 128, d) * (4 if more else 8)
+
+
+# GEMM1 unsplit with room for the W_o conversion in its side warp: GEMM2 is split in four or not at all, never in two
+@pytest.mark.parametrize("d,tiles2,split2", [(512, 0.2, 4), (512, 0.24, 1), (512, 0.4, 1), (1024, 0.24, 1)])
+def test_output_projection_is_not_split_in_two_beside_a_side_warp(d, tiles2, split2):
+    rows = int(sms() * tiles2) // (d // 256)
+    case = W.merge_case(780 + rows, vocab=500, d=d, h=4, n_spans=rows * 128 - 5, kmin=4, kmax=4)
+    ran = check(case)
+    t1 = tiles(case.token_ids.numel(), d)
+    assert ran["gemm1"] == min(t1, sms())
+    assert ran["gemm2"] == tiles(rows * 128, d) * split2
+    assert ran["w_o"] == 0   # no conversion kernel: in the split product or in GEMM1's side warp

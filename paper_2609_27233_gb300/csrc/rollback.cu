@@ -310,7 +310,8 @@ __device__ __forceinline__ void fence_proxy_async_global() {
   asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
-template <int D, bool ROPE>
+// ROPE: key rows that a warp rotates at once (0: none are rotated)
+template <int D, int ROPE>
 __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs a, PlanArrays arr, PageDesc pd) {
   constexpr int ROW = D * 2;                 // bytes of one entry of one (K|V, head)
   constexpr int TILE = kPageSize * ROW;      // bytes of a unit
@@ -464,26 +465,33 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
   // arithmetic is packed; four rows' words are read ahead.  Consecutive rows with
   // the same shift (a run of moved entries between two spans) reuse the angles.
   // With single bf16 elements (pairs l and l + 32) the long context's move took
-  // 111 us against 95 us now (75 us without rotation).
+  // 111 us against 95 us now (75 us without rotation).  Where 16 lanes hold a row
+  // (rotary_dim <= 64), each half of the warp takes a row of its own: 300 sequences
+  // of 4096 entries at D = 64 took 637 us with half of the lanes idle, 482 now (a
+  // choice made in the kernel cost whole rows of D = 128 one to two percent).
   static_assert(D / 2 <= 64, "two pairs per lane");
   auto rotate_rows = [&](const Unit &m, uint8_t *stage) {
-    const int half = a.rotary_dim / 2;   // even
-    const bool mine = 2 * lane < half;
+    constexpr int rows = ROPE > 1 ? ROPE : 1;
+    const int half = a.rotary_dim / 2;   // a multiple of 8
+    const int l = lane % (32 / rows), mine_of = lane / (32 / rows);
+    const bool mine = 2 * l < half;
     float prev = 0.f;
     float2 sn = make_float2(0.f, 0.f), cs = make_float2(1.f, 1.f);
-    for (int r0 = m.ra; r0 < m.rb; r0 += 4) {
+    for (int r0 = m.ra; r0 < m.rb; r0 += 4 * rows) {
       uint32_t x[4], y[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const uint32_t *row = reinterpret_cast<const uint32_t *>(stage + min(r0 + u, m.rb - 1) * ROW);
-        x[u] = mine ? row[lane] : 0u;
-        y[u] = mine ? row[half / 2 + lane] : 0u;
+        const uint32_t *row =
+            reinterpret_cast<const uint32_t *>(stage + min(r0 + u * rows + mine_of, m.rb - 1) * ROW);
+        x[u] = mine ? row[l] : 0u;
+        y[u] = mine ? row[half / 2 + l] : 0u;
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const int r = r0 + u;
-        if (r >= m.rb) break;
-        const float rf = (float)__shfl_sync(0xffffffffu, m.shift, r);
+        if (r0 + u * rows >= m.rb) break;
+        const int r = r0 + u * rows + mine_of;
+        const int32_t shift = __shfl_sync(0xffffffffu, m.shift, rows == 1 ? r : min(r, m.rb - 1));
+        const float rf = rows == 1 || r < m.rb ? (float)shift : 0.f;
         if (rf == 0.f) continue;   // a surrogate or an entry that keeps its position
         if (rf != prev) {
           auto angle = [&](float w, float &s_out, float &c_out) {
@@ -498,7 +506,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
             c_out = fmaf(-err, sn0, cs0);
           };
           if (mine) {
-            const float2 w = *reinterpret_cast<const float2 *>(s_w + 2 * lane);
+            const float2 w = *reinterpret_cast<const float2 *>(s_w + 2 * l);
             angle(w.x, sn.x, cs.x);
             angle(w.y, sn.y, cs.y);
           }
@@ -512,8 +520,8 @@ __global__ void __launch_bounds__(kBulkThreads, 1) rollback_bulk_kernel(MoveArgs
           const float2 yr = __ffma2_rn(yv, cs, make_float2(-xs.x, -xs.y));
           const __nv_bfloat162 xo = __floats2bfloat162_rn(xr.x, xr.y), yo = __floats2bfloat162_rn(yr.x, yr.y);
           uint32_t *row = reinterpret_cast<uint32_t *>(stage + r * ROW);
-          row[lane] = *reinterpret_cast<const uint32_t *>(&xo);
-          row[half / 2 + lane] = *reinterpret_cast<const uint32_t *>(&yo);
+          row[l] = *reinterpret_cast<const uint32_t *>(&xo);
+          row[half / 2 + l] = *reinterpret_cast<const uint32_t *>(&yo);
         }
       }
     }
@@ -683,8 +691,9 @@ umim_status kv_rollback(const umim_paged_kv *kv, int32_t *block_table, int32_t m
   ma.rope_inv_freq = rope_inv_freq;
   ma.rotary_dim = rope_inv_freq ? rotary_dim : 0;
   const bool rope = rope_inv_freq != nullptr;
-  auto kern = rope ? (D == 128 ? rollback_bulk_kernel<128, true> : rollback_bulk_kernel<64, true>)
-                   : (D == 128 ? rollback_bulk_kernel<128, false> : rollback_bulk_kernel<64, false>);
+  auto kern = !rope ? (D == 128 ? rollback_bulk_kernel<128, 0> : rollback_bulk_kernel<64, 0>)
+              : D == 64 ? rollback_bulk_kernel<64, 2>
+                        : (rotary_dim <= 64 ? rollback_bulk_kernel<128, 2> : rollback_bulk_kernel<128, 1>);
   const int threads = kBulkThreads;
   const int smem = kBulkMovers * kBulkStages * kPageSize * D * 2;
   if (!allow_smem(kern, smem)) return UMIM_ERR_CUDA;

@@ -1219,7 +1219,9 @@ umim_status prefill_attention(const void *q, const void *k, const void *v, int T
   auto vk = plan ? (D == 128 ? vt_kernel<128, true> : vt_kernel<64, true>)
                  : (D == 128 ? vt_kernel<128, false> : vt_kernel<64, false>);
   const int64_t vt_blocks = a.Tp / kPfKeys * Hkv;
-  // eight CTAs an SM are resident (six took 82 us for 96 000 rows of 8 heads, eight 71)
+  // eight CTAs an SM are launched: five (D = 128) or six (64) of them are resident by
+  // their registers, the others follow as those finish (with six an SM in all, 96 000
+  // rows of 8 heads took 82 us, with eight 71)
   const unsigned vt_grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(vt_blocks, 8LL * std::max(num_sms, 1)));
   if (launch_pdl(vk, dim3(vt_grid), dim3(kPfVtThreads), plan ? 2 * sizeof(int32_t) * ((size_t)B + 1) : 0, stream, a) !=
       cudaSuccess)

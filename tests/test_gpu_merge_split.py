@@ -1,5 +1,6 @@
-"""The merge module's products with K split over a cluster: every split (8, 4, 2, none) of both products, at the
-edges of the 128-row tiles, against the float64 oracle (the tolerance of every merge test)."""
+"""The merge module's products with K split over a cluster, at the edges of the 128-row tiles, against the float64
+oracle (the tolerance of every merge test).  The splits named below are those of 152 SMs; that a size takes the split it
+should is checked in test_gpu_merge_paths.py."""
 import pytest
 import torch
 

@@ -14,7 +14,7 @@
 // plan kernel before every call cost 3 us of a call of 16 (four sequences of
 // 24 000 entries: rollback and attention 178.3 -> 175.8 us).
 //
-// Per warp: a private ring of NST stages; lane 0 issues TMA tensor loads of
+// Per warp: a private ring of NST stages; an elected lane issues TMA tensor loads of
 // whole pages (K and V tiles of 16 x D bf16, 128-byte swizzled) into the
 // ring and each stage completes an mbarrier.  S = Q K^T (G <= 16 query heads
 // as the M=16 side) and O += P V run as mma.sync m16n8k16 on operands read

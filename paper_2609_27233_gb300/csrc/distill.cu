@@ -456,7 +456,7 @@ __device__ __forceinline__ void st_async_f4(uint32_t raddr, float4 v, uint32_t r
 // One cluster of C CTAs per student row; CTA `rank` owns vectors
 // [rank * chunk_vecs, ...) of the row.  T compute threads (NW warps) hold
 // KV vectors of the teacher and student row each, and one more warp issues
-// the copies: lane 0 walks the CTA's paired rows, waits for a stage of the
+// the copies: an elected lane walks the CTA's paired rows, waits for a stage of the
 // ring to be released by every compute warp, and loads the teacher and
 // student chunk into it with two bulk copies.
 //

@@ -325,9 +325,10 @@ __global__ void gather_rows_kernel(const uint4 *table, int64_t vocab, const int3
 // columns of the tile, adding the CTAs' parts over distributed shared memory
 // in rank order, and finishes them (bias, GELU, stores, statistics per 32
 // columns, merged by rank 0).  Eight lanes read one 128-byte line of a peer:
-// with one row per lane instead the reduction alone took about 20 us.  Measured over the whole call (with the next
-// paragraph and the early weights below): 13 spans at d = 4096 100.9 -> 54.0 us,
-// one prompt's 238 spans 119 -> 94 us (with its compressed prompt).
+// with one row per lane instead the reduction alone took about 20 us.  Measured
+// over the whole call (with the next paragraph, the early weights below and LN_o's
+// CTA per row): 13 spans at d = 4096 99.7 -> 36.5 us, one prompt's 238 spans 118 ->
+// 86 us (with its compressed prompt).
 // CONV: B is bf16 and A fp16 (the output projection); eight warps turn each
 // staged B tile into fp16 (times kWoScale, exact) in place before its MMAs, so
 // no fp16 copy of W_o is written and read back.

@@ -31,9 +31,11 @@
 //
 // V is transposed first (per sequence, padded to a multiple of 64 keys) so
 // that both products read K-major operands and every TMA copy starts on a
-// 16-byte boundary.  A plan kernel turns cu_seqlens into per-sequence tile
-// offsets and padded key offsets (and validates them); tiles run heaviest
-// (last in their sequence) first.
+// 16-byte boundary.  The transposing CTAs turn cu_seqlens into per-sequence tile
+// offsets and padded key offsets (and validate them) in shared memory, each for
+// itself, and write every query tile's record; beyond kPfSmemBatch sequences a plan
+// kernel ahead of them derives the offsets.  Tiles run heaviest (last in their
+// sequence) first.
 #include <cuda_fp16.h>
 
 #include "common.cuh"

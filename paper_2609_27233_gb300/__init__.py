@@ -65,7 +65,7 @@ def lib():
 # for a ctypes struct), and the current stream's handle is read without
 # building a Stream object (0.2 us against 2.9 us).  A step of five
 # calls (cache update, four layers' attention) over three short sequences, bound
-# by the host, went from 152 to 94 us.
+# by the host, went from 137-148 to 85-93 us (with one launch less a call).
 def _p(t):
     return None if t is None else t.data_ptr()
 

@@ -44,3 +44,31 @@ def test_scores_of_nan_and_minus_infinity(call, value, lo, hi, hq, d):
     else:
         float_close(got[0], want[0])
     float_close(got[1], want[1])
+
+
+@pytest.mark.parametrize("value", ["nan", "-inf"])
+@pytest.mark.parametrize("hq,hkv,d", [(32, 8, 128), (16, 8, 64), (7, 1, 128)])   # two heads at a time, and one
+def test_prefill_scores_of_nan_and_minus_infinity(value, hq, hkv, d):
+    """One key of the middle of a sequence, the last one of another: rows from it on are NaN, or weigh it 0; rows before
+    it, the other heads' and the other sequences' rows (in the same tiles of keys) are untouched."""
+    m, dv = umim(), dev()
+    lens = [300, 70, 515, 129] + [260] * {32: 16, 16: 30, 7: 1}[hq]
+    T, cu_np = sum(lens), np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert (hq // hkv % 2 == 0 and 2 * (T // 128 + len(lens)) * (hq // 2) >= 7 * sms) == (hq > 7)
+    # (V of a quarter, as in the other edge tests: the output's rounding stays below the absolute tolerance)
+    q, k, v = (W.bf16_normal((T, h, d), s, 950 + i, dv) for i, (h, s) in enumerate(((hq, 1.0), (hkv, 1.0), (hkv, 0.25))))
+    q[:, :, 0] = q[:, :, 0].abs() + 0.5
+    hit = [int(cu_np[2]) + 197, int(cu_np[2]) - 1]
+    for t in hit:
+        k[t, 0, 0] = float(value)
+    status = m.new_status(dv)
+    out = m.umim_prefill_attention(q, k, v, torch.from_numpy(cu_np).to(dv), dev_status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    want = oracle.prefill_attention(W.bits(q), W.bits(k), W.bits(v), cu_np)
+    got = out.cpu().double().numpy()
+    nan = np.isnan(want)
+    assert nan.any() == (value == "nan")
+    np.testing.assert_array_equal(np.isnan(got), nan)
+    float_close(np.where(nan, 0.0, got), np.where(nan, 0.0, want))
